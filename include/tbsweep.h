@@ -352,8 +352,9 @@ TB_API void tb_server_destroy(tb_server* server);
  * passes, 1 row-0 writer, 2 last-row reduction, 3 finalisation, 4 narrow
  * (whole boundary in shared memory), 5 open-plan join, 6 open-plan late
  * crossings. bytes[c] is the algorithmic HBM traffic of those launches: a
- * pass or a join reads and writes every boundary entry once (16 bytes per
- * entry), the writer writes 8, the reduction reads 8, a late crossing reads
+ * pass reads and writes every entry of the tiles it visits once (16 bytes per
+ * entry; tiles that the plan knows to be exactly zero are not visited), a join
+ * every boundary entry, the writer writes 8, the reduction reads 8, a late crossing reads
  * two entries and writes one (24 bytes per output entry). */
 #define TB_PROFILE_CLASSES 7
 typedef struct {

@@ -330,8 +330,9 @@ int run_device(const Plan& P, const uint8_t* d_bits, int64_t nb, void* d_ws, int
                 tp.B = boundary;
                 tp.b_stride = b_stride;
                 tp.h = P.h; tp.lo = d.lo; tp.n = xstride;
-                tp.tile_shift = P.h - P.tc_wb - TC_VEC_BITS;
+                tp.tile_shift = P.h - P.tc_wb - TC_VEC_BITS - d.skip.n;
                 tp.ntiles = (int64_t)nbat << tp.tile_shift;
+                tp.skip = d.skip;
                 tp.mat = mats + d.mat;
                 tp.steps = steps;
                 tp.pre = d.pre;
@@ -344,7 +345,7 @@ int run_device(const Plan& P, const uint8_t* d_bits, int64_t nb, void* d_ws, int
                 tp.fault = fault;
                 tp.selftest = t_tc_selftest ? 1 : 0;
                 const int grid = (int)std::min<int64_t>(tp.ntiles, (int64_t)TC_CTAS_PER_SM * nsm);
-                ProfScope ps(PC_PASS, 16.0 * (double)nbat * (double)b_stride, st);
+                ProfScope ps(PC_PASS, 16.0 * (double)nbat * (double)(b_stride >> d.skip.n), st);
                 TB_CUDA(launch_tc_pass(P.opts.precision, tp, grid, st));
             }
         }
@@ -352,8 +353,9 @@ int run_device(const Plan& P, const uint8_t* d_bits, int64_t nb, void* d_ws, int
             const PassDesc& d = P.passes[k];
             PassParams pp;
             pp.h = P.h; pp.lo = d.lo; pp.n = xstride;
-            pp.tile_shift = P.h - TILE_BITS;
+            pp.tile_shift = P.h - TILE_BITS - d.skip.n;
             pp.ntiles = (int64_t)nbat << pp.tile_shift;
+            pp.skip = d.skip;
             pp.steps = pass_steps + d.pstep0;
             pp.xs_step0 = d.xs_step[0]; pp.xs_q0 = d.xs_q[0];
             pp.xs_step1 = d.xs_step[1]; pp.xs_q1 = d.xs_q[1];
@@ -368,7 +370,7 @@ int run_device(const Plan& P, const uint8_t* d_bits, int64_t nb, void* d_ws, int
             const int rc = encode_pass_map(&tmap, d, boundary, P.h, nbat);
             if (rc != TB_OK) return rc;
             const int grid = (int)std::min<int64_t>(pp.ntiles, (int64_t)PASS_CTAS_PER_SM * nsm);  // persistent CTAs
-            ProfScope ps(PC_PASS, 16.0 * (double)nbat * (double)b_stride, st);
+            ProfScope ps(PC_PASS, 16.0 * (double)nbat * (double)(b_stride >> d.skip.n), st);
             TB_CUDA(launch_pass(d, pp, tmap, grid, st));
         }
 

@@ -145,7 +145,10 @@ int tb_batch_create(const tb_batch_item* items, int nitems, void* d_ws, int64_t 
         if (!small_path(items[i].plan->p) && items[i].nb > 0) wide.push_back(i);
     auto cost = [&](int i) {
         const Plan& P = items[i].plan->p;
-        return (double)items[i].nb * (double)(P.n_pass_launches() + 2) * std::ldexp(1.0, P.h);
+        double visited = 2.0;  // boundary sweeps: row-0 writer and reduction, then the tiles each pass visits
+        for (const PassDesc& d : P.passes) visited += std::ldexp(1.0, -d.skip.n);
+        for (const TcPass& d : P.tc_passes) visited += std::ldexp(1.0, -d.skip.n);
+        return (double)items[i].nb * visited * std::ldexp(1.0, P.h);
     };
     std::sort(wide.begin(), wide.end(), [&](int a, int b) { return cost(a) > cost(b); });
     std::vector<std::vector<int>> branch(nbranches);

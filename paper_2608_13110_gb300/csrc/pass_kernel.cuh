@@ -52,8 +52,9 @@ namespace tb {
 
 struct PassParams {
     int h, lo, n;
-    int tile_shift;       // log2(tiles per batch element) = h - TILE_BITS
+    int tile_shift;       // log2(tiles visited per batch element) = h - TILE_BITS - skip.n
     int64_t ntiles;       // nbatch << tile_shift
+    TileSkip skip;        // which tiles are visited
     const StepG* steps;   // the pass's first step
     int xs_step0, xs_q0, xs_step1, xs_q1;
     const uint8_t* bits;  // bitstring of batch element b at bits + b*n
@@ -586,18 +587,20 @@ __device__ __forceinline__ void tma_store_tile(const CUtensorMap* m, int c3, int
 __device__ __forceinline__ void tma_wait_read_all() { asm volatile("cp.async.bulk.wait_group.read 0;\n" ::: "memory"); }
 __device__ __forceinline__ void tma_wait_all() { asm volatile("cp.async.bulk.wait_group 0;\n" ::: "memory"); }
 
-// Tensor-map coordinates (dimensions 3 and 4) of global tile gt. Windows at
-// bit 0: dimension 3 is the global tile index. Other windows: dimension 3 =
-// the address bits between the low bits and the window, dimension 4 = the
-// bits above the window and the batch element.
+// Tensor-map coordinates (dimensions 3 and 4) of visited tile gt (the whole
+// producer warp, col = this lane's column of the tile map). Windows at bit 0:
+// dimension 3 is the tile index with the batch element. Other windows:
+// dimension 3 = the address bits between the low bits and the window,
+// dimension 4 = the bits above the window and the batch element.
 template <class SH>
-__device__ __forceinline__ void tile_coords(const PassParams& p, int64_t gt, int& c3, int& c4) {
+__device__ __forceinline__ void tile_coords(const PassParams& p, int64_t gt, uint32_t col, uint32_t lane, int& c3,
+                                            int& c4) {
+    const int64_t b = gt >> p.tile_shift;
+    const int64_t t = tile_of_warp(p.skip.base, col, lane, (uint32_t)(gt & (((int64_t)1 << p.tile_shift) - 1)));
     if constexpr (SH::BOT) {
-        c3 = (int)gt;
+        c3 = (int)((b << (p.h - TILE_BITS)) + t);
         c4 = 0;
     } else {
-        const int64_t b = gt >> p.tile_shift;
-        const int64_t t = gt & (((int64_t)1 << p.tile_shift) - 1);
         const int nl = p.lo - SH::C;
         c3 = (int)(t & (((int64_t)1 << nl) - 1));
         c4 = (int)((b << (p.h - p.lo - SH::M)) + (t >> nl));
@@ -614,7 +617,7 @@ constexpr int pass_smem_bytes() {
 
 template <int TYPE, int M>
 __global__ void __launch_bounds__(PASS_THREADS, PASS_CTAS_PER_SM)
-    pass_kernel(const PassParams p, const __grid_constant__ CUtensorMap tmap) {
+    pass_kernel(const __grid_constant__ PassParams p, const __grid_constant__ CUtensorMap tmap) {
     using SH = Shape<TYPE, M>;
     static_assert(SH::valid(), "invalid pass shape");
     static_assert(SH::NS <= XM_HIGH_BIT, "variant mask: one bit per step, bit XM_HIGH_BIT for the four-variant step");
@@ -629,60 +632,74 @@ __global__ void __launch_bounds__(PASS_THREADS, PASS_CTAS_PER_SM)
     const uint32_t full0 = pass_smem_u32(bars), done0 = full0 + 8 * PASS_STAGES;
     const uint32_t stage0 = pass_smem_u32(stages);
 
-    stage_coefficients<SH>(p.steps, sc, tid);
-    if (tid == 0) {
-        for (int s = 0; s < PASS_STAGES; ++s) {
-            pbar_init(full0 + 8 * s, 1);
-            pbar_init(done0 + 8 * s, PASS_CONSUMERS / 32);
-        }
-        *s_abort = 0;
-        asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
-    }
-    __syncthreads();
-
     const int64_t first = blockIdx.x;
     const int64_t ntl = first < p.ntiles ? (p.ntiles - 1 - first) / gridDim.x + 1 : 0;  // tiles of this CTA
     const uint32_t tries = p.selftest ? PASS_SELFTEST_TRIES : PASS_WAIT_TRIES;
+    const uint32_t lane = tid & 31u;
+    const uint32_t col = tile_col(p.skip, lane);
+    int t3[PASS_STAGES], t4[PASS_STAGES];  // producer: coordinates of the tile in each stage
+
+    // The producer warp (the first of the last warpgroup) works on tile
+    // coordinates together; its lane 0 sets the barriers up and issues every
+    // copy. The first loads start before the coefficients are staged.
+    if ((tid >> 5) == PASS_CONSUMERS / 32) {
+        if (lane == 0) {
+            asm volatile("prefetch.tensormap [%0];\n" ::"l"(reinterpret_cast<uint64_t>(&tmap)) : "memory");
+            for (int s = 0; s < PASS_STAGES; ++s) {
+                pbar_init(full0 + 8 * s, 1);
+                pbar_init(done0 + 8 * s, PASS_CONSUMERS / 32);
+            }
+            *s_abort = 0;
+            asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+            asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+        }
+        if (!p.selftest)
+            for (int k = 0; k < ntl && k < PASS_STAGES; ++k) {
+                tile_coords<SH>(p, first + (int64_t)k * gridDim.x, col, lane, t3[k], t4[k]);
+                if (lane == 0) {
+                    pbar_expect_tx(full0 + 8 * k, TILE_BYTES);
+                    tma_load_tile(stage0 + (uint32_t)k * TILE_BYTES, &tmap, t3[k], t4[k], full0 + 8 * k);
+                }
+            }
+    }
+    stage_coefficients<SH>(p.steps, sc, tid);
+    __syncthreads();
 
     static_assert(PASS_THREADS - PASS_CONSUMERS == 128, "one producer warpgroup");
     static_assert((PASS_THREADS - PASS_CONSUMERS) * PASS_PRODUCER_REGS + PASS_CONSUMERS * PASS_CONSUMER_REGS <=
                       PASS_THREADS * (65536 / PASS_THREADS / 8 * 8),
                   "register split exceeds the launch's registers");
     if (tid >= PASS_CONSUMERS) {
-        // ---------------- producer: one thread of the last warpgroup
+        // ---------------- producer: one warp of the last warpgroup
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;\n" ::"n"(PASS_PRODUCER_REGS));
-        if (tid != PASS_CONSUMERS) return;
-        asm volatile("prefetch.tensormap [%0];\n" ::"l"(reinterpret_cast<uint64_t>(&tmap)) : "memory");
+        if ((tid >> 5) != PASS_CONSUMERS / 32) return;
         int64_t last_load[PASS_STAGES];  // tile index k of the latest load per stage (-1: none)
-        for (int st = 0; st < PASS_STAGES; ++st) last_load[st] = -1;
-        if (!p.selftest) {
-            for (int64_t k = 0; k < ntl && k < PASS_STAGES; ++k) {
-                int c3, c4;
-                tile_coords<SH>(p, first + k * gridDim.x, c3, c4);
-                pbar_expect_tx(full0 + 8 * (int)k, TILE_BYTES);
-                tma_load_tile(stage0 + (uint32_t)k * TILE_BYTES, &tmap, c3, c4, full0 + 8 * (int)k);
-                last_load[k] = k;
-            }
-        }
+        for (int st = 0; st < PASS_STAGES; ++st) last_load[st] = !p.selftest && st < ntl ? st : -1;
         int s = 0;
         uint32_t ph = 0;
         for (int64_t k = 0; k < ntl; ++k) {
-            if (!pbar_wait(done0 + 8 * s, ph, tries)) {
-                if (atomicExch(s_abort, 1) == 0) atomicAdd(p.fault, 1);
+            int n3 = 0, n4 = 0;  // the stage's next tile, worked out while the consumers are busy
+            if (k + PASS_STAGES < ntl) tile_coords<SH>(p, first + (k + PASS_STAGES) * gridDim.x, col, lane, n3, n4);
+            const bool gave_up = !pbar_wait(done0 + 8 * s, ph, tries);
+            if (__any_sync(0xffffffffu, gave_up)) {
+                if (lane == 0 && atomicExch(s_abort, 1) == 0) atomicAdd(p.fault, 1);
                 break;
             }
-            int c3, c4;
-            tile_coords<SH>(p, first + k * gridDim.x, c3, c4);
-            tma_store_tile(&tmap, c3, c4, stage0 + (uint32_t)s * TILE_BYTES);
-            if (k + PASS_STAGES < ntl) {
-                tma_wait_read_all();  // the store has read the stage
-                tile_coords<SH>(p, first + (k + PASS_STAGES) * gridDim.x, c3, c4);
-                pbar_expect_tx(full0 + 8 * s, TILE_BYTES);
-                tma_load_tile(stage0 + (uint32_t)s * TILE_BYTES, &tmap, c3, c4, full0 + 8 * s);
-                last_load[s] = k + PASS_STAGES;
+            if (lane == 0) {
+                tma_store_tile(&tmap, t3[s], t4[s], stage0 + (uint32_t)s * TILE_BYTES);
+                if (k + PASS_STAGES < ntl) {
+                    tma_wait_read_all();  // the store has read the stage
+                    pbar_expect_tx(full0 + 8 * s, TILE_BYTES);
+                    tma_load_tile(stage0 + (uint32_t)s * TILE_BYTES, &tmap, n3, n4, full0 + 8 * s);
+                    last_load[s] = k + PASS_STAGES;
+                    t3[s] = n3;
+                    t4[s] = n4;
+                }
             }
+            __syncwarp();
             if (++s == PASS_STAGES) { s = 0; ph ^= 1u; }
         }
+        if (lane != 0) return;
         tma_wait_all();
         if (*(volatile int*)s_abort) {
             // loads still in flight must land before the CTA's shared memory goes
@@ -705,15 +722,10 @@ __global__ void __launch_bounds__(PASS_THREADS, PASS_CTAS_PER_SM)
     int s = 0;
     uint32_t ph = 0;
     for (int64_t k = 0; k < ntl; ++k) {
-        const bool gave_up = !pbar_wait(full0 + 8 * s, ph, tries);
-        if (__any_sync(0xffffffffu, gave_up)) {  // the whole warp stops
-            if ((tid & 31u) == 0 && atomicExch(s_abort, 1) == 0) atomicAdd(p.fault, 1);
-            break;
-        }
         const int64_t gt = first + k * gridDim.x;
         const int64_t b = gt >> p.tile_shift;
         const int64_t t = gt & tmask;
-        if (b != cur_b) {  // per-bitstring state, read once per batch element
+        if (b != cur_b) {  // per-bitstring state, read once per batch element while the tile is on its way
             if (cur_b >= 0) flush_max(runmax, p.maxs + cur_b * p.sstride + p.slot + 1);
             runmax = 0.0f;
             cur_b = b;
@@ -723,6 +735,11 @@ __global__ void __launch_bounds__(PASS_THREADS, PASS_CTAS_PER_SM)
             xmask = 0;
             if (p.xs_step0 >= 0) xmask |= (xb[p.xs_q0] ? 1u : 0u) << p.xs_step0;
             if (p.xs_step1 >= 0) xmask |= (xb[p.xs_q1] ? 1u : 0u) << p.xs_step1;
+        }
+        const bool gave_up = !pbar_wait(full0 + 8 * s, ph, tries);
+        if (__any_sync(0xffffffffu, gave_up)) {  // the whole warp stops
+            if ((tid & 31u) == 0 && atomicExch(s_abort, 1) == 0) atomicAdd(p.fault, 1);
+            break;
         }
         if (t == 0 && tid == 0) p.exps[b * p.sstride + p.slot + 1] = cur_s;
 

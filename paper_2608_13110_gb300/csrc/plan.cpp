@@ -80,6 +80,8 @@ M2 clifford(int k) {
     return m2_mul(P[k % 4], R[k / 4]);
 }
 
+static bool is_bottom(int type) { return type == P_BOT || type == P_BOT_START || type == P_BOT_END; }
+
 static float2 f2(cd z) { return make_float2((float)z.real(), (float)z.imag()); }
 
 // ---------------------------------------------------------------------------
@@ -279,6 +281,155 @@ static void build_pass_steps(Plan& P) {
                 }
             for (int e = 0; e < BLK_ENTRIES; ++e) P.pass_steps.push_back(blk[e]);
         }
+    }
+}
+
+// ---------------------------------------------------------------------------
+// Tiles of exact zeros (TileSkip)
+// ---------------------------------------------------------------------------
+// A monomial one-qubit gate (I, S, a Pauli, T times any of them: a third of
+// the random Cliffords) copies or flips a value, so the boundary is exactly
+// zero wherever the stored bits disagree with it: two monomial gates between
+// stored layers p-1 and p fix the parity of address bits p-1 and p (one chance
+// in nine per bit), and nothing later in the sweep undoes that before one of
+// the two bits is summed out. Support holds the affine space over GF(2) that
+// contains every nonzero entry: equations parity(address & mask) = value.
+// What it saves is the tiles no pass reads, computes or writes: with random
+// Clifford + T gates a pass visits 0.39-0.43 of its tiles at width 31, 0.44-0.52
+// at 28, 0.66-0.73 at 20, 0.9 at 16 (n = 70, d = 56, two bitstrings: 311 ms
+// visiting every tile, 134 ms; n = 30, d = 40, 32 bitstrings: 7.47 and 5.29 ms);
+// circuits without monomial gates visit every tile as before.
+class Support {
+public:
+    static constexpr int TMP = 63;  // variable of the bit a step sums out
+
+    // Add an equation (dependent ones are dropped).
+    void add(uint64_t mask, int value) {
+        for (const Eq& e : eq_)
+            if (mask >> e.pivot & 1) { mask ^= e.mask; value ^= e.value; }
+        if (!mask) return;
+        const int pv = 63 - __builtin_clzll(mask);
+        for (Eq& e : eq_)
+            if (e.mask >> pv & 1) { e.mask ^= mask; e.value ^= value; }
+        eq_.push_back(Eq{mask, value, pv});
+    }
+
+    // Project a variable out.
+    void eliminate(int var) {
+        int hit = -1;
+        for (size_t i = 0; i < eq_.size(); ++i)
+            if (eq_[i].mask >> var & 1) hit = (int)i;
+        if (hit < 0) return;
+        const Eq h = eq_[hit];
+        std::vector<Eq> old;
+        old.swap(eq_);
+        for (size_t i = 0; i < old.size(); ++i)
+            if ((int)i != hit) {
+                const bool has = (old[i].mask >> var & 1) != 0;
+                add(has ? old[i].mask ^ h.mask : old[i].mask, has ? old[i].value ^ h.value : old[i].value);
+            }
+    }
+
+    // One paired step: target bit t (s summed out, a' created), control bit c
+    // or -1. nz[c][a'][s]: the step's coefficient is not exactly zero.
+    void step(int t, int c, const bool (&nz)[2][2][2]) {
+        const uint64_t tb = (uint64_t)1 << t, sb = (uint64_t)1 << TMP, cb = c < 0 ? 0 : (uint64_t)1 << c;
+        for (Eq& e : eq_)
+            if (e.mask & tb) { e.mask ^= tb | sb; e.pivot = TMP; }
+        std::vector<Eq> old;  // pivots moved with the rename: rebuild
+        old.swap(eq_);
+        for (const Eq& e : old) add(e.mask, e.value);
+        for (int m = 1; m < 8; ++m) {  // equations that every nonzero coefficient satisfies
+            if ((m & 4) && c < 0) continue;
+            int seen = 0;  // bit v: parity v occurs
+            for (int i = 0; i < 8; ++i) {
+                if (c < 0 && (i & 4)) continue;
+                if (nz[i >> 2][i >> 1 & 1][i & 1]) seen |= 1 << __builtin_parity(i & m);
+            }
+            if (seen == 1 || seen == 2)
+                add(((m & 4) ? cb : 0) | ((m & 2) ? tb : 0) | ((m & 1) ? sb : 0), seen == 2);
+        }
+        eliminate(TMP);
+    }
+
+    // The tiles a pass visits: outside[i] is the address bit of tile-index bit
+    // i, in ascending order.
+    TileSkip skip(const std::vector<int>& outside, int h) const {
+        Support s = *this;
+        uint64_t out = 0;
+        for (int b : outside) out |= (uint64_t)1 << b;
+        for (int b = 0; b < h; ++b)
+            if (!(out >> b & 1)) s.eliminate(b);
+        TileSkip k;
+        std::memset(&k, 0, sizeof(k));
+        const int nb = (int)outside.size();
+        auto index_mask = [&](uint64_t m) {
+            uint32_t r = 0;
+            for (int i = 0; i < nb; ++i)
+                if (m >> outside[i] & 1) r |= (uint32_t)1 << i;
+            return r;
+        };
+        // reduced equations: each pivot bit is determined by bits that are no pivots
+        uint32_t pivots = 0;
+        for (const Eq& e : s.eq_) {
+            const uint32_t pv = index_mask((uint64_t)1 << e.pivot);
+            pivots |= pv;
+            if (e.value) k.base |= pv;
+            ++k.n;
+        }
+        for (int i = 0, u = 0; i < nb; ++i) {
+            if (pivots >> i & 1) continue;
+            k.col[u] = (uint32_t)1 << i;
+            for (const Eq& e : s.eq_)
+                if (e.mask >> outside[i] & 1) k.col[u] |= index_mask((uint64_t)1 << e.pivot);
+            ++u;
+        }
+        return k;
+    }
+
+private:
+    struct Eq {
+        uint64_t mask;
+        int value, pivot;  // pivot: the highest variable, in no other equation
+    };
+    std::vector<Eq> eq_;
+};
+
+// Fill in every pass's TileSkip. row0: the support of the row-0 boundary.
+static void tile_skips(Plan& P, Support s) {
+    const int h = P.h;
+    bool finite = true;  // 0 x inf is not 0: such gates leave every tile visited
+    for (const auto& g : P.steps64)
+        for (const cd& z : g)
+            if (!std::isfinite(z.real()) || !std::isfinite(z.imag())) finite = false;
+    int done = 0;
+    auto advance = [&](int end) {
+        for (; done < end; ++done) {
+            bool nz[2][2][2];
+            for (int i = 0; i < 8; ++i)  // of either output bit's variant
+                nz[i >> 2][i >> 1 & 1][i & 1] = P.steps64[done][i] != 0.0 || P.steps64[done][8 + i] != 0.0;
+            s.step(P.step_tgt[done], P.step_ctl[done], nz);
+        }
+    };
+    if (!finite) s = Support();
+    std::vector<int> outside;
+    for (PassDesc& d : P.passes) {
+        const int C = is_bottom(d.type) ? TILE_BITS : TILE_BITS - d.M;  // low address bits of a tile
+        outside.clear();
+        for (int b = C; b < h; ++b)
+            if (is_bottom(d.type) || b < d.lo || b >= d.lo + d.M) outside.push_back(b);
+        if ((int)outside.size() > MAX_TILE_BITS) continue;  // wider than the device evaluates
+        if (finite) advance(d.step0);
+        d.skip = s.skip(outside, h);
+    }
+    for (TcPass& d : P.tc_passes) {
+        outside.clear();
+        for (int b = 0, below = 0; b < h; ++b)
+            if (b < d.lo || b >= d.lo + P.tc_wb)
+                if (below++ >= TC_VEC_BITS) outside.push_back(b);
+        if ((int)outside.size() > MAX_TILE_BITS) continue;
+        if (finite) advance(d.step0);
+        d.skip = s.skip(outside, h);
     }
 }
 
@@ -503,6 +654,17 @@ int plan_build(Plan& P, int n, int d, const uint8_t* cliff, const uint8_t* tmask
         for (int p = 1; p < k; ++p) v *= Mp[p].a[((s >> p) & 1) * 2 + ((s >> (p - 1)) & 1)];
         P.init_low[s] = f2(v);
     }
+    Support row0;  // where the row-0 boundary is not zero
+    {
+        auto fixed = [](cd a, cd b) { return (a == 0.0) != (b == 0.0); };
+        const cd* a0 = U(0, 0).a;
+        if (fixed(a0[0], a0[2])) row0.add(1, a0[0] == 0.0);
+        for (int p = 1; p < h; ++p) {
+            const cd* g = Mp[p].a;  // [s_p][s_(p-1)]
+            if (fixed(g[0], g[1]) && fixed(g[2], g[3]) && fixed(g[0], g[2]))
+                row0.add((uint64_t)3 << (p - 1), g[0] == 0.0);
+        }
+    }
     P.init_mid.assign((size_t)2 << m, make_float2(0, 0));
     for (int b = 0; b < 2; ++b)
         for (int64_t s = 0; s < ((int64_t)1 << m); ++s) {
@@ -631,6 +793,7 @@ int plan_build(Plan& P, int n, int d, const uint8_t* cliff, const uint8_t* tmask
         if (P.passes.empty()) { err = "no pass schedule fits these window limits"; return TB_EINVAL; }
         build_pass_steps(P);
     }
+    tile_skips(P, row0);
 
     sym_alg1(n, d, &P.width, &P.log2cost);
     if (P.open_k > 0) {

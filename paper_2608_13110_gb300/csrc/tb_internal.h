@@ -108,6 +108,43 @@ struct StepG {
 };
 static_assert(sizeof(StepG) == 16 * sizeof(float2), "StepG entries are read as raw float2 arrays");
 
+// Tiles a pass visits. Monomial one-qubit gates leave exact zeros in the
+// boundary: the planner tracks which parities of address bits are fixed
+// wherever the boundary is not zero (plan.cpp: tile_skips), and a pass visits
+// only the tiles whose outside address bits satisfy the parities among them.
+// The other tiles are zero before the pass and stay zero, and every boundary
+// buffer holds those zeros explicitly (the row-0 writer writes all entries),
+// so leaving them alone changes no value. A pass's tile index t numbers the
+// address bits outside its tile in ascending order; n of its bits are
+// determined by the others, and the visited tiles u = 0 .. 2^(bits-n)-1 are
+// t = tile_of(u), an affine map over GF(2): base XOR the columns of u's set
+// bits. A warp evaluates it with one column per lane and one XOR reduction
+// (the loop form below costs one thread 2 us per pass when the code and the
+// arguments are cold: 0.58 against 0.52 ms for a whole width-18 amplitude).
+constexpr int MAX_TILE_BITS = 24;
+struct TileSkip {
+    int n;
+    uint32_t base;
+    uint32_t col[MAX_TILE_BITS];
+};
+
+inline uint32_t tile_of(const TileSkip& k, uint32_t u) {
+    uint32_t t = k.base;
+    for (int i = 0; i < MAX_TILE_BITS; ++i)
+        if (u >> i & 1) t ^= k.col[i];
+    return t;
+}
+
+#ifdef __CUDACC__
+// All 32 lanes, u uniform; col = this lane's column (tile_col).
+__device__ __forceinline__ uint32_t tile_col(const TileSkip& k, uint32_t lane) {
+    return lane < MAX_TILE_BITS ? k.col[lane] : 0u;
+}
+__device__ __forceinline__ uint32_t tile_of_warp(uint32_t base, uint32_t col, uint32_t lane, uint32_t u) {
+    return base ^ __reduce_xor_sync(0xffffffffu, (u >> lane & 1u) ? col : 0u);
+}
+#endif
+
 // Host-side description of one pass (launch arguments).
 struct PassDesc {
     int type;
@@ -118,6 +155,7 @@ struct PassDesc {
     int nsteps;    // pass_nsteps(type, M)
     int xs_step[2];  // bit of the pass's variant mask set by an output bit, -1 if none
     int xs_q[2];     // the qubit whose output bit sets it
+    TileSkip skip;   // tiles visited
 };
 
 // ---- Tensor-core dense blocks (TB_PRECISION_TF32X3 / TB_PRECISION_BF16X3) --
@@ -152,6 +190,7 @@ struct TcPass {
     int64_t mat;   // byte offset of the pass's split matrix in the tc_mats table
     int step0;     // contiguous steps covered (pre, block, post)
     int nsteps;
+    TileSkip skip;  // tiles visited
 };
 
 // Bytes of one split matrix (hi then lo) of a dense block over WB bits.

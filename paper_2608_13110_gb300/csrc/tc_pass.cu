@@ -132,7 +132,7 @@ __device__ __forceinline__ void reg_step(float2 (&v)[NV], const float2* g, int c
 }
 
 template <int KIND>
-__global__ void __launch_bounds__(TC_THREADS, TC_CTAS_PER_SM) tc_pass_kernel(const TcParams p) {
+__global__ void __launch_bounds__(TC_THREADS, TC_CTAS_PER_SM) tc_pass_kernel(const __grid_constant__ TcParams p) {
     using C = TcCfg<KIND>;
     constexpr int NV = C::NV;
     extern __shared__ __align__(16) uint8_t dsm[];
@@ -171,10 +171,12 @@ __global__ void __launch_bounds__(TC_THREADS, TC_CTAS_PER_SM) tc_pass_kernel(con
 
     const int lo = p.lo;
     const int64_t lomask = ((int64_t)1 << lo) - 1;
+    const uint32_t tcol = tile_col(p.skip, tid & 31);
     const int64_t tmask = ((int64_t)1 << p.tile_shift) - 1;
     auto vec_addr = [&](int64_t gt) {  // entry 0 of this thread's vector in tile gt
         const int64_t b = gt >> p.tile_shift;
-        const int64_t u = ((gt & tmask) << TC_VEC_BITS) | tid;
+        const int64_t t = tile_of_warp(p.skip.base, tcol, tid & 31, (uint32_t)(gt & tmask));
+        const int64_t u = (t << TC_VEC_BITS) | tid;
         return b * p.b_stride + (u & lomask) + ((u >> lo) << (lo + C::WB));
     };
     auto load_vec = [&](float2 (&v)[NV], int64_t a0) {

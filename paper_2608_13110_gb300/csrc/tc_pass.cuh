@@ -14,8 +14,9 @@ struct TcParams {
     float2* B;              // boundary of batch element 0
     int64_t b_stride;       // complex entries between batch elements
     int h, lo, n;
-    int tile_shift;         // log2(tiles per batch element) = h - WB - TC_VEC_BITS
+    int tile_shift;         // log2(tiles visited per batch element) = h - WB - TC_VEC_BITS - skip.n
     int64_t ntiles;         // nbatch << tile_shift
+    TileSkip skip;          // which tiles are visited
     const uint8_t* mat;     // the pass's split matrix: hi part, then lo part
     const StepG* steps;     // the plan's step array
     TcStep pre, post;       // register steps around the block (t < 0: none)
