@@ -257,12 +257,10 @@ int run_device(const Plan& P, const uint8_t* d_bits, int64_t nb, void* d_ws, int
         SmallParams sp;
         sp.n = P.n;
         sp.h = P.h;
+        sp.nsm = num_sms();
         sp.bits = d_bits;
         sp.steps = tab<StepG>(d_ws, L.steps);
-        sp.tgt = tab<int8_t>(d_ws, L.step_tgt);
-        sp.ctl = tab<int8_t>(d_ws, L.step_ctl);
         sp.xq = tab<int16_t>(d_ws, L.step_xq);
-        sp.row_end = tab<int32_t>(d_ws, L.row_end);
         sp.nrows = (int)P.row_end.size();
         sp.init_low = tab<float2>(d_ws, L.init_low);
         sp.init_top = tab<float2>(d_ws, L.init_top);

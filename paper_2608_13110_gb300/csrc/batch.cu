@@ -120,10 +120,7 @@ int tb_batch_create(const tb_batch_item* items, int nitems, void* d_ws, int64_t 
         si.p.nb = (int)items[i].nb;
         si.p.bits = items[i].d_bits;
         si.p.steps = at<StepG>(base, T.steps);
-        si.p.tgt = at<int8_t>(base, T.step_tgt);
-        si.p.ctl = at<int8_t>(base, T.step_ctl);
         si.p.xq = at<int16_t>(base, T.step_xq);
-        si.p.row_end = at<int32_t>(base, T.row_end);
         si.p.nrows = (int)P.row_end.size();
         si.p.init_low = at<float2>(base, T.init_low);
         si.p.init_top = at<float2>(base, T.init_top);

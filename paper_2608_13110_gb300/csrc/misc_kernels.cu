@@ -2,6 +2,8 @@
 // kernel (arXiv 2608.13110, Sec. 3.1, Algorithm 1).
 #include "misc_kernels.cuh"
 
+#include <algorithm>
+
 namespace tb {
 
 __device__ __forceinline__ float2 cmul(float2 a, float2 b) {
@@ -211,90 +213,484 @@ cudaError_t launch_finalize(const FinalizeParams& p, cudaStream_t st) {
 }
 
 // ---------------------------------------------------------------------------
-// Narrow boundaries (h <= 12): one CTA per bitstring keeps B in shared memory
-// for the whole sweep: row 0, every paired step of rows 1..n-2 in order, the
-// last-row contraction; power-of-two rescaling after every row.
+// Narrow boundaries (h <= 12): one CTA per bitstring runs the whole sweep, row
+// 0, every paired step of rows 1..n-2 in order, the last-row contraction, with
+// the boundary on chip. Every step evaluates, for both of its outputs,
+//   re = fma(g0r, ar, fma(-g0i, ai, fma(g1r, br, -g1i br))), a = in[s=0], b = in[s=1]
+// (and im alike), whatever the layout below.
 // ---------------------------------------------------------------------------
-__device__ float block_max_f(float v, float* red) {
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, off));
-    const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-    __syncthreads();
-    if (l == 0) red[w] = v;
-    __syncthreads();
-    float m = 0.0f;
-    for (int i = 0; i < (int)(blockDim.x >> 5); ++i) m = fmaxf(m, red[i]);
-    return m;
-}
 
-__device__ int small_rescale(float2* Bs, int N, float* red) {
-    float m = 0.0f;
-    for (int e = threadIdx.x; e < N; e += blockDim.x) m = fmaxf(m, fmaxf(fabsf(Bs[e].x), fabsf(Bs[e].y)));
-    m = block_max_f(m, red);
-    const int s = rescale_exp_m(m);
-    const float sc = ldexpf(1.0f, s);
-    for (int e = threadIdx.x; e < N; e += blockDim.x) Bs[e] = make_float2(Bs[e].x * sc, Bs[e].y * sc);
-    __syncthreads();
-    return s;
-}
-
-// Bitstring b of one narrow plan, the whole sweep in shared memory (Bs holds
-// 2^h entries).
-__device__ void small_sweep(const SmallParams& p, int b, float2* Bs, float* redf, double2* redd) {
-    const uint8_t* xb = p.bits + (int64_t)b * p.n;
-    const int h = p.h, N = 1 << h;
-    const int x0 = xb[0] ? 1 : 0;
-    for (int e = threadIdx.x; e < N; e += blockDim.x)
-        Bs[e] = cmul(p.init_low[e], p.init_top[x0 * 2 + ((e >> (h - 1)) & 1)]);
-    __syncthreads();
-    long long S = small_rescale(Bs, N, redf);
-    int step = 0;
-    for (int row = 0; row < p.nrows; ++row) {
-        for (; step < p.row_end[row]; ++step) {
-            const int t = p.tgt[step], u = p.ctl[step], q = p.xq[step];
-            const int var = (q >= 0 && xb[q]) ? 1 : 0;
-            const float2* g = p.steps[step].g[var];
-            for (int i = threadIdx.x; i < (N >> 1); i += blockDim.x) {
-                const int i0 = ((i >> t) << (t + 1)) | (i & ((1 << t) - 1));
-                const int i1 = i0 | (1 << t);
-                const int c = u >= 0 ? (i0 >> u) & 1 : 0;
-                const float2* gg = g + 4 * c;
-                const float2 a = Bs[i0], bb = Bs[i1];
-                Bs[i0] = cmac2m(gg[0], a, gg[1], bb);
-                Bs[i1] = cmac2m(gg[2], a, gg[3], bb);
-            }
-            __syncthreads();
+// --- 8 <= h <= 12: register windows ----------------------------------------
+// A thread holds 2^(RW+1) entries in registers: RW consecutive address bits
+// (the window) and one spectator bit v whose two values share a packed pair
+// (paired FP32 FMA, coefficients broadcast). The steps whose targets lie in
+// the window are register arithmetic; the boundary goes through shared memory
+// only when the window moves. The targets walk 0..h-1 and back, so the windows
+// at the two ends serve the steps before and after the turn: per two rows four
+// windows (h = 12, RW = 4: 8 + 4 + 8 + 4 steps) where every single step used
+// to read and write shared memory behind a barrier. What bounds it: FP32 issue
+// (8 FMA per entry and step) once every SM has two warps per scheduler, the
+// chain of window moves and steps below that. n = 45, us for 1 / 256 / 2048
+// bitstrings, one step per barrier -> this form: width 8 147 / 154 / 458 ->
+// 49 / 49 / 109, width 10 240 / 279 / 1234 -> 62 / 82 / 434, width 11
+// 365 / 456 / 2353 -> 101 / 135 / 807, width 12 604 / 817 / 4771 -> 144 / 237 / 1770.
+// Power-of-two rescaling (exact) at every turn, folded into the next window's
+// first coefficients.
+template <int H, int RW>
+struct Narrow {
+    static constexpr int T = 1 << (H - RW - 1);  // threads
+    static constexpr int NK = 1 << RW;           // packed pairs per thread
+    static constexpr int MID = H - 2 * RW;       // bits between the two turn windows
+    static constexpr int NW = (T + 31) / 32;
+    // spectator bit of the window [lo, lo + RW): neither in it nor next to it,
+    // and not among the lowest bits, which the lanes hold
+    static constexpr int vbit(int lo) { return lo + RW + 1 <= H - 1 ? H - 1 : lo - 2; }
+    // shared-memory slot: 16 lanes that differ in the four lowest address bits
+    // outside any window fall into 16 different 8-byte banks
+    static constexpr uint32_t swz(uint32_t a) { return a ^ ((a >> RW) & 15u); }
+    // thread bits fill the address bits other than the window's and v, ascending
+    __device__ static __forceinline__ uint32_t thread_addr(int lo, uint32_t t) {
+        const int v = vbit(lo), below = v < lo ? v : lo;
+        uint32_t a = t & ((1u << below) - 1u);
+        t >>= below;
+        if (v < lo) {  // bit lo - 1 above v
+            a |= (t & 1u) << (lo - 1);
+            t >>= 1;
         }
-        S += small_rescale(Bs, N, redf);
+        return a | (t << (lo + RW));
+    }
+};
+
+constexpr int NARROW_CF = 24;  // packed coefficients per step: [c][g00r g00i -g00i g01r .. -g11i]
+
+__device__ __forceinline__ float2 nfma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+
+template <int N>
+__device__ __forceinline__ void narrow_cf(float2 (&c)[N], const float2* src) {
+    const float4* s4 = reinterpret_cast<const float4*>(src);
+#pragma unroll
+    for (int i = 0; i < N / 2; ++i) {
+        const float4 q = s4[i];
+        c[2 * i] = make_float2(q.x, q.y);
+        c[2 * i + 1] = make_float2(q.z, q.w);
+    }
+}
+
+// Step on register bit K; CK: control register bit, -1: cf holds the block of
+// this thread's control value (or the step has no control).
+template <bool SC, int NK, int K, int CK>
+__device__ __forceinline__ void narrow_step(float2 (&P)[NK], float2 (&Q)[NK], const float2* cf, float s) {
+#pragma unroll
+    for (int cv = 0; cv < (CK >= 0 ? 2 : 1); ++cv) {
+        float2 c[12];
+        narrow_cf(c, cf + 12 * cv);
+        if constexpr (SC) {
+#pragma unroll
+            for (int i = 0; i < 12; ++i) c[i] = __fmul2_rn(c[i], make_float2(s, s));
+        }
+#pragma unroll
+        for (int k = 0; k < NK; ++k) {
+            if (k & (1 << K)) continue;
+            if (CK >= 0 && ((k >> (CK < 0 ? 0 : CK)) & 1) != cv) continue;
+            const int k1 = k | (1 << K);
+            const float2 aP = P[k], aQ = Q[k], bP = P[k1], bQ = Q[k1];
+            P[k] = nfma2(c[0], aP, nfma2(c[2], aQ, nfma2(c[3], bP, __fmul2_rn(c[5], bQ))));
+            Q[k] = nfma2(c[0], aQ, nfma2(c[1], aP, nfma2(c[3], bQ, __fmul2_rn(c[4], bP))));
+            P[k1] = nfma2(c[6], aP, nfma2(c[8], aQ, nfma2(c[9], bP, __fmul2_rn(c[11], bQ))));
+            Q[k1] = nfma2(c[6], aQ, nfma2(c[7], aP, nfma2(c[9], bQ, __fmul2_rn(c[10], bP))));
+        }
+    }
+}
+
+// SC: the coefficients of the first step carry the rescale s.
+// Forward targets T0 .. T0+N-1 (register bits of the window at lo); cf: the
+// row's coefficients, step of target t at cf + t * NARROW_CF.
+template <bool SC, int NK, int LO, int T0, int N>
+__device__ __forceinline__ void narrow_fwd(float2 (&P)[NK], float2 (&Q)[NK], const float2* cf, uint32_t addr, float s) {
+    if constexpr (N > 0) {
+        const float2* c = cf + T0 * NARROW_CF;
+        if constexpr (T0 == LO) {
+            if (T0 > 0 && ((addr >> (T0 > 0 ? T0 - 1 : 0)) & 1u)) c += 12;
+            narrow_step<SC, NK, 0, -1>(P, Q, c, s);
+        } else {
+            narrow_step<SC, NK, T0 - LO, T0 - LO - 1>(P, Q, c, s);
+        }
+        narrow_fwd<false, NK, LO, T0 + 1, N - 1>(P, Q, cf, addr, 1.0f);
+    }
+}
+
+// Reversed targets T0, T0-1, .. (N of them); step of target t at cf + (H-1-t) * NARROW_CF.
+template <bool SC, int NK, int RW, int H, int LO, int T0, int N>
+__device__ __forceinline__ void narrow_rev(float2 (&P)[NK], float2 (&Q)[NK], const float2* cf, uint32_t addr, float s) {
+    if constexpr (N > 0) {
+        const float2* c = cf + (H - 1 - T0) * NARROW_CF;
+        if constexpr (T0 == LO + RW - 1) {
+            if (T0 < H - 1 && ((addr >> (T0 + 1)) & 1u)) c += 12;
+            narrow_step<SC, NK, T0 - LO, -1>(P, Q, c, s);
+        } else {
+            narrow_step<SC, NK, T0 - LO, T0 - LO + 1>(P, Q, c, s);
+        }
+        narrow_rev<false, NK, RW, H, LO, T0 - 1, N - 1>(P, Q, cf, addr, 1.0f);
+    }
+}
+
+template <int H, int RW>
+struct NarrowRun {
+    using W = Narrow<H, RW>;
+    static constexpr int NK = W::NK, T = W::T;
+    static constexpr int ROW_CF = H * NARROW_CF;       // a row's packed coefficients
+    static constexpr int CYCLE = 2 * H * 8;            // raw coefficients of two rows
+    static constexpr int PRE = (CYCLE + T - 1) / T;    // of which a thread stages this many
+    float2* Bs;
+    float2* cf;     // [2 buffers][2 rows][H][NARROW_CF]
+    float* red;     // [2][NW]
+    const SmallParams& p;
+    const uint8_t* xb;
+    uint32_t t;
+    long long S;
+    float2 pre[PRE];
+
+    __device__ __forceinline__ void sync() const {
+        if constexpr (T <= 32) __syncwarp(T == 32 ? 0xffffffffu : (1u << T) - 1u);
+        else asm volatile("bar.sync 1, %0;" ::"n"(T) : "memory");
+    }
+    // coefficients of rows 2 cyc and 2 cyc + 1: global memory -> registers -> shared memory
+    __device__ __forceinline__ void fetch(int cyc) {
+#pragma unroll
+        for (int i = 0; i < PRE; ++i) {
+            const int w = i * T + (int)t, st = 2 * H * cyc + (w >> 3);
+            if (w < CYCLE && st < p.nrows * H) {
+                const int q = p.xq[st];
+                pre[i] = p.steps[st].g[q >= 0 && xb[q] ? 1 : 0][w & 7];
+            }
+        }
+    }
+    __device__ __forceinline__ void stage(int cyc) {
+        float2* dst = cf + (cyc & 1) * 2 * ROW_CF;
+#pragma unroll
+        for (int i = 0; i < PRE; ++i) {
+            const int w = i * T + (int)t;
+            if (w < CYCLE) {
+                float2* o = dst + (w >> 3) * NARROW_CF + 3 * (w & 7);
+                o[0] = make_float2(pre[i].x, pre[i].x);
+                o[1] = make_float2(pre[i].y, pre[i].y);
+                o[2] = make_float2(-pre[i].y, -pre[i].y);
+            }
+        }
+    }
+    template <int LO>
+    __device__ __forceinline__ uint32_t addr() const { return W::thread_addr(LO, t); }
+    template <int LO>
+    __device__ __forceinline__ void load(float2 (&P)[NK], float2 (&Q)[NK]) const {
+        const uint32_t b = W::swz(addr<LO>());
+#pragma unroll
+        for (int k = 0; k < NK; ++k) {
+            const float2 lo = Bs[b ^ W::swz((uint32_t)k << LO)];
+            const float2 hi = Bs[b ^ W::swz((uint32_t)k << LO) ^ W::swz(1u << W::vbit(LO))];
+            P[k] = make_float2(lo.x, hi.x);
+            Q[k] = make_float2(lo.y, hi.y);
+        }
+    }
+    template <int LO>
+    __device__ __forceinline__ void store(const float2 (&P)[NK], const float2 (&Q)[NK]) const {
+        const uint32_t b = W::swz(addr<LO>());
+#pragma unroll
+        for (int k = 0; k < NK; ++k) {
+            Bs[b ^ W::swz((uint32_t)k << LO)] = make_float2(P[k].x, Q[k].x);
+            Bs[b ^ W::swz((uint32_t)k << LO) ^ W::swz(1u << W::vbit(LO))] = make_float2(P[k].y, Q[k].y);
+        }
+    }
+    // this turn's maximum, for the scale every thread takes after the next sync
+    __device__ __forceinline__ void put_max(float m, int turn) {
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, off));
+        if ((t & 31) == 0) red[(turn & 1) * W::NW + (t >> 5)] = m;
+    }
+    __device__ __forceinline__ float reg_max(const float2 (&P)[NK], const float2 (&Q)[NK]) const {
+        float m = 0.0f;
+#pragma unroll
+        for (int k = 0; k < NK; ++k)
+            m = fmaxf(m, fmaxf(fmaxf(fabsf(P[k].x), fabsf(P[k].y)), fmaxf(fabsf(Q[k].x), fabsf(Q[k].y))));
+        return m;
+    }
+    __device__ __forceinline__ float take_scale(int turn) {
+        float m = 0.0f;
+#pragma unroll
+        for (int i = 0; i < W::NW; ++i) m = fmaxf(m, red[(turn & 1) * W::NW + i]);
+        const int s = rescale_exp_m(m);
+        S += s;
+        return ldexpf(1.0f, s);
+    }
+    // targets of the middle windows, RW at a time; the first one is rescaled
+    template <bool SC, int T0>
+    __device__ __forceinline__ void mid_fwd(const float2* c, float s) {
+        if constexpr (T0 < H - RW) {
+            constexpr int N = (H - RW - T0) < RW ? (H - RW - T0) : RW;
+            float2 P[NK], Q[NK];
+            load<T0>(P, Q);
+            narrow_fwd<SC, NK, T0, T0, N>(P, Q, c, addr<T0>(), s);
+            store<T0>(P, Q);
+            sync();
+            mid_fwd<false, T0 + N>(c, 1.0f);
+        }
+    }
+    template <bool SC, int T0>
+    __device__ __forceinline__ void mid_rev(const float2* c, float s) {
+        if constexpr (T0 >= RW) {
+            constexpr int N = (T0 - RW + 1) < RW ? (T0 - RW + 1) : RW;
+            constexpr int LO = T0 - RW + 1;
+            float2 P[NK], Q[NK];
+            load<LO>(P, Q);
+            narrow_rev<SC, NK, RW, H, LO, T0, N>(P, Q, c, addr<LO>(), s);
+            store<LO>(P, Q);
+            sync();
+            mid_rev<false, T0 - N>(c, 1.0f);
+        }
+    }
+
+    __device__ void run(int b, double2* redd) {
+        constexpr int N = 1 << H, TOP = H - RW;
+        const int x0 = xb[0] ? 1 : 0;
+        float m = 0.0f;
+        fetch(0);
+        for (int e = (int)t; e < N; e += T) {
+            const float2 v = cmul(p.init_low[e], p.init_top[x0 * 2 + ((e >> (H - 1)) & 1)]);
+            Bs[W::swz((uint32_t)e)] = v;
+            m = fmaxf(m, fmaxf(fabsf(v.x), fabsf(v.y)));
+        }
+        stage(0);
+        put_max(m, 0);
+        sync();
+        int row = 0, turn = 0;
+        float s = take_scale(0);
+        if (p.nrows > 0) {
+            float2 P[NK], Q[NK];
+            load<0>(P, Q);
+#pragma unroll
+            for (int k = 0; k < NK; ++k) {
+                P[k] = __fmul2_rn(P[k], make_float2(s, s));
+                Q[k] = __fmul2_rn(Q[k], make_float2(s, s));
+            }
+            for (int cyc = 0;; ++cyc) {
+                const float2* c = cf + (cyc & 1) * 2 * ROW_CF;
+                fetch(cyc + 1);
+                narrow_fwd<false, NK, 0, 0, RW>(P, Q, c, 0u, 1.0f);
+                put_max(reg_max(P, Q), ++turn);
+                store<0>(P, Q);
+                sync();
+                s = take_scale(turn);
+                if constexpr (W::MID > 0) mid_fwd<true, RW>(c, s);
+                load<TOP>(P, Q);
+                narrow_fwd<W::MID == 0, NK, TOP, TOP, RW>(P, Q, c, addr<TOP>(), s);
+                if (++row == p.nrows) {
+                    put_max(reg_max(P, Q), ++turn);
+                    store<TOP>(P, Q);
+                    break;
+                }
+                narrow_rev<false, NK, RW, H, TOP, H - 1, RW>(P, Q, c + ROW_CF, 0u, 1.0f);
+                put_max(reg_max(P, Q), ++turn);
+                store<TOP>(P, Q);
+                stage(cyc + 1);
+                sync();
+                s = take_scale(turn);
+                if constexpr (W::MID > 0) mid_rev<true, H - RW - 1>(c + ROW_CF, s);
+                load<0>(P, Q);
+                narrow_rev<W::MID == 0, NK, RW, H, 0, RW - 1, RW>(P, Q, c + ROW_CF, addr<0>(), s);
+                if (++row == p.nrows) {
+                    put_max(reg_max(P, Q), ++turn);
+                    store<0>(P, Q);
+                    break;
+                }
+            }
+            sync();
+            s = take_scale(turn);
+        }
+        const int xl = xb[p.n - 1] ? 1 : 0;
+        double ar = 0.0, ai = 0.0;
+        for (int e = (int)t; e < N; e += T) {
+            const float2 z = Bs[W::swz((uint32_t)e)];
+            const float2 v = cmul(make_float2(z.x * s, z.y * s), p.red_low[2 * e + xl]);
+            ar += (double)v.x;
+            ai += (double)v.y;
+        }
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) {
+            ar += __shfl_xor_sync(0xffffffffu, ar, off);
+            ai += __shfl_xor_sync(0xffffffffu, ai, off);
+        }
+        if ((t & 31) == 0) redd[t >> 5] = make_double2(ar, ai);
+        sync();
+        if (t == 0) {
+            double2 tot = redd[0];
+            for (int i = 1; i < W::NW; ++i) { tot.x += redd[i].x; tot.y += redd[i].y; }
+            const int Si = (int)max(-1000000LL, min(1000000LL, S));
+            p.out[2 * b] = scalbn(tot.x, -Si);
+            p.out[2 * b + 1] = scalbn(tot.y, -Si);
+        }
+    }
+};
+
+// --- h <= 7: one warp, address bits 0..4 on the lanes, the rest in registers --
+// A step on a lane bit takes the partner's entry by shuffle; each lane loads
+// the coefficient row of its own output one row ahead, so the steps wait for
+// nothing but their own chain (n = 12, d = 8, 64 bitstrings, whole host call:
+// 73 us with a CTA and a barrier per step, 54 us).
+template <int H>
+__device__ void narrow_warp(const SmallParams& p, int b) {
+    constexpr int LB = H < 5 ? H : 5, R = H > 5 ? 1 << (H - 5) : 1;
+    const uint32_t lane = threadIdx.x & 31u;
+    const uint8_t* xb = p.bits + (int64_t)b * p.n;
+    const bool live = lane < (1u << LB);
+    float2 v[R];
+    const int x0 = xb[0] ? 1 : 0;
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        const uint32_t e = (lane & ((1u << LB) - 1u)) | ((uint32_t)r << LB);
+        v[r] = live ? cmul(p.init_low[e], p.init_top[x0 * 2 + ((e >> (H - 1)) & 1)]) : make_float2(0.f, 0.f);
+    }
+    long long S = 0;
+    auto rescale = [&]() {
+        float m = 0.0f;
+#pragma unroll
+        for (int r = 0; r < R; ++r) m = fmaxf(m, fmaxf(fabsf(v[r].x), fabsf(v[r].y)));
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, off));
+        const int s = rescale_exp_m(m);
+        const float sc = ldexpf(1.0f, s);
+#pragma unroll
+        for (int r = 0; r < R; ++r) v[r] = make_float2(v[r].x * sc, v[r].y * sc);
+        S += s;
+    };
+    rescale();
+    // coefficients of one row: for every target, this lane's output rows. A
+    // register target or control needs more than one: [register control or
+    // target value][2 entries]
+    constexpr int NC = R > 1 ? 4 : 1;
+    float4 cur[H][NC], nxt[H][NC];
+    auto fetch = [&](int row, float4 (&o)[H][NC]) {
+        if (row >= p.nrows) return;
+        const bool fwd = (row & 1) == 0;  // row 0 here is the circuit's row 1
+#pragma unroll
+        for (int tg = 0; tg < H; ++tg) {
+            const int st = row * H + (fwd ? tg : H - 1 - tg);
+            const int q = p.xq[st];
+            const float4* g = reinterpret_cast<const float4*>(p.steps[st].g[q >= 0 && xb[q] ? 1 : 0]);
+            const int ct = fwd ? tg - 1 : tg + 1;  // control bit (outside 0..H-1: none)
+            const bool cin = ct >= 0 && ct < H;
+#pragma unroll
+            for (int i = 0; i < NC; ++i) {
+                const int ap = tg < LB ? (int)(lane >> tg & 1u) : (i & 1);
+                const int c = !cin ? 0 : ct < LB ? (int)(lane >> (ct < 0 ? 0 : ct) & 1u) : (i >> 1);
+                o[tg][i] = g[c * 2 + ap];
+            }
+        }
+    };
+    auto out = [](float4 g, float2 a, float2 bb) {
+        return cmac2m(make_float2(g.x, g.y), a, make_float2(g.z, g.w), bb);
+    };
+    auto step = [&](int tg, int ct, const float4 (&g)[NC]) {
+        if (tg < LB) {
+            const bool hi = (lane >> tg & 1u) != 0;
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                float2 o;
+                o.x = __shfl_xor_sync(0xffffffffu, v[r].x, 1 << tg);
+                o.y = __shfl_xor_sync(0xffffffffu, v[r].y, 1 << tg);
+                const int c = (ct >= LB && ct < H) ? (r >> (ct - LB)) & 1 : 0;  // register control
+                v[r] = out(g[NC > 1 ? 2 * c : 0], hi ? o : v[r], hi ? v[r] : o);
+            }
+        } else {
+            const int K = tg - LB;
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                if (r & (1 << K)) continue;
+                const int r1 = (r | (1 << K)) & (R - 1);
+                const int c = (ct >= LB && ct < H) ? (r >> (ct - LB)) & 1 : 0;
+                const float2 a = v[r], bb = v[r1];
+                v[r] = out(g[NC > 1 ? 2 * c : 0], a, bb);
+                v[r1] = out(g[NC > 1 ? 2 * c + 1 : 0], a, bb);
+            }
+        }
+    };
+    fetch(0, cur);
+    for (int row = 0; row < p.nrows; ++row) {
+        fetch(row + 1, nxt);
+        if ((row & 1) == 0) {
+#pragma unroll
+            for (int tg = 0; tg < H; ++tg) step(tg, tg - 1, cur[tg]);
+        } else {
+#pragma unroll
+            for (int tg = H - 1; tg >= 0; --tg) step(tg, tg + 1, cur[tg]);
+        }
+        rescale();
+#pragma unroll
+        for (int tg = 0; tg < H; ++tg)
+#pragma unroll
+            for (int i = 0; i < NC; ++i) cur[tg][i] = nxt[tg][i];
     }
     const int xl = xb[p.n - 1] ? 1 : 0;
     double ar = 0.0, ai = 0.0;
-    for (int e = threadIdx.x; e < N; e += blockDim.x) {
-        const float2 v = cmul(Bs[e], p.red_low[2 * e + xl]);
-        ar += (double)v.x;
-        ai += (double)v.y;
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        const uint32_t e = (lane & ((1u << LB) - 1u)) | ((uint32_t)r << LB);
+        const float2 w = live ? cmul(v[r], p.red_low[2 * e + xl]) : make_float2(0.f, 0.f);
+        ar += (double)w.x;
+        ai += (double)w.y;
     }
-    const double2 tot = block_sum_d2(make_double2(ar, ai), redd);
-    if (threadIdx.x == 0) {
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+        ar += __shfl_xor_sync(0xffffffffu, ar, off);
+        ai += __shfl_xor_sync(0xffffffffu, ai, off);
+    }
+    if (lane == 0) {
         const int Si = (int)max(-1000000LL, min(1000000LL, S));
-        p.out[2 * b] = scalbn(tot.x, -Si);
-        p.out[2 * b + 1] = scalbn(tot.y, -Si);
+        p.out[2 * b] = scalbn(ar, -Si);
+        p.out[2 * b + 1] = scalbn(ai, -Si);
     }
 }
 
-__global__ void __launch_bounds__(SMALL_THREADS) small_kernel(const SmallParams p) {
-    extern __shared__ float2 Bs[];
-    __shared__ float redf[SMALL_THREADS / 32];
-    __shared__ double2 redd[SMALL_THREADS / 32];
-    small_sweep(p, blockIdx.x, Bs, redf, redd);
+// Window bits at width h. few: the bitstrings fit one CTA per SM, so the length
+// of one sweep counts (fewer entries per thread, more warps); otherwise the
+// FP32 pipe counts (more steps per window). Measured with 1 / 256 / 512
+// bitstrings at n = 45 (us, before the last refinements): width 11 with RW = 2
+// 109 / 180 / 349, 3 124 / 151 / 308; width 12 with RW = 3 164 / 322 / 634,
+// 4 195 / 259 / 538; at widths 8 to 10 RW = 2 is the best for both (width 10:
+// 70 / 91 / 154, RW = 3 117 / 122 / 167).
+constexpr int narrow_rw(int h, bool few) { return h <= 10 ? 2 : h == 11 ? (few ? 2 : 3) : (few ? 3 : 4); }
+constexpr int narrow_threads(int h, bool few) { return h < 8 ? 32 : 1 << (h - narrow_rw(h, few) - 1); }
+constexpr int narrow_smem(int h, bool few) {  // boundary, coefficients, reduction scratch of every warp
+    return h < 8 ? 0 : (8 << h) + 2 * 2 * h * NARROW_CF * 8 + (narrow_threads(h, few) / 32) * 24;
+}
+
+template <int H, bool FEW>
+__device__ __forceinline__ void narrow_sweep(const SmallParams& p, int b, uint8_t* smem) {
+    if constexpr (H < 8) {
+        if (threadIdx.x < 32) narrow_warp<H>(p, b);
+    } else {
+        using R = NarrowRun<H, narrow_rw(H, FEW)>;
+        static_assert(R::T >= 32, "whole warps");
+        if (threadIdx.x >= R::T) return;
+        float2* Bs = reinterpret_cast<float2*>(smem);
+        float2* cf = Bs + (1 << H);
+        double2* redd = reinterpret_cast<double2*>(cf + 2 * 2 * R::ROW_CF);  // [NW], then red [2][NW]
+        R r{Bs, cf, reinterpret_cast<float*>(redd + R::W::NW), p, p.bits + (int64_t)b * p.n, threadIdx.x, 0, {}};
+        r.run(b, redd);
+    }
+}
+
+template <int H, bool FEW>
+__global__ void __launch_bounds__(narrow_threads(H, FEW)) narrow_kernel(const __grid_constant__ SmallParams p) {
+    extern __shared__ __align__(16) uint8_t nsm[];
+    narrow_sweep<H, FEW>(p, blockIdx.x, nsm);
 }
 
 // Several narrow plans in one launch: block i evaluates bitstring
 // i - first_block of the item whose block range holds i.
-__global__ void __launch_bounds__(SMALL_THREADS) small_multi_kernel(const SmallItem* items, int nitems) {
-    extern __shared__ float2 Bs[];
-    __shared__ float redf[SMALL_THREADS / 32];
-    __shared__ double2 redd[SMALL_THREADS / 32];
+constexpr int NARROW_MULTI_THREADS = 128;
+static_assert(narrow_threads(12, false) <= NARROW_MULTI_THREADS && narrow_threads(11, false) <= NARROW_MULTI_THREADS &&
+                  narrow_threads(10, false) <= NARROW_MULTI_THREADS, "one CTA size for every width");
+__global__ void __launch_bounds__(NARROW_MULTI_THREADS) narrow_multi_kernel(const SmallItem* items, int nitems) {
+    extern __shared__ __align__(16) uint8_t nsm[];
     int lo = 0, hi = nitems - 1;
     const int64_t blk = blockIdx.x;
     while (lo < hi) {  // last item with first_block <= blk
@@ -303,19 +699,54 @@ __global__ void __launch_bounds__(SMALL_THREADS) small_multi_kernel(const SmallI
         else hi = mid - 1;
     }
     const SmallParams p = items[lo].p;
-    small_sweep(p, (int)(blk - items[lo].first_block), Bs, redf, redd);
+    const int b = (int)(blk - items[lo].first_block);
+    switch (p.h) {
+        case 1: narrow_sweep<1, false>(p, b, nsm); break;
+        case 2: narrow_sweep<2, false>(p, b, nsm); break;
+        case 3: narrow_sweep<3, false>(p, b, nsm); break;
+        case 4: narrow_sweep<4, false>(p, b, nsm); break;
+        case 5: narrow_sweep<5, false>(p, b, nsm); break;
+        case 6: narrow_sweep<6, false>(p, b, nsm); break;
+        case 7: narrow_sweep<7, false>(p, b, nsm); break;
+        case 8: narrow_sweep<8, false>(p, b, nsm); break;
+        case 9: narrow_sweep<9, false>(p, b, nsm); break;
+        case 10: narrow_sweep<10, false>(p, b, nsm); break;
+        case 11: narrow_sweep<11, false>(p, b, nsm); break;
+        case 12: narrow_sweep<12, false>(p, b, nsm); break;
+        default: break;
+    }
 }
 
 cudaError_t launch_small_multi(const SmallItem* d_items, int nitems, int64_t nblocks, int hmax, cudaStream_t st) {
-    const int smem = (1 << hmax) * (int)sizeof(float2);
-    small_multi_kernel<<<(unsigned)nblocks, SMALL_THREADS, smem, st>>>(d_items, nitems);
+    int smem = 0;
+    for (int h = 1; h <= hmax; ++h) smem = std::max(smem, narrow_smem(h, false));
+    narrow_multi_kernel<<<(unsigned)nblocks, NARROW_MULTI_THREADS, smem, st>>>(d_items, nitems);
+    return cudaGetLastError();
+}
+
+template <int H>
+cudaError_t launch_narrow(const SmallParams& p, cudaStream_t st) {
+    if (p.nb <= p.nsm) narrow_kernel<H, true><<<p.nb, narrow_threads(H, true), narrow_smem(H, true), st>>>(p);
+    else narrow_kernel<H, false><<<p.nb, narrow_threads(H, false), narrow_smem(H, false), st>>>(p);
     return cudaGetLastError();
 }
 
 cudaError_t launch_small(const SmallParams& p, cudaStream_t st) {
-    const int smem = (1 << p.h) * (int)sizeof(float2);
-    small_kernel<<<p.nb, SMALL_THREADS, smem, st>>>(p);
-    return cudaGetLastError();
+    switch (p.h) {
+        case 1: return launch_narrow<1>(p, st);
+        case 2: return launch_narrow<2>(p, st);
+        case 3: return launch_narrow<3>(p, st);
+        case 4: return launch_narrow<4>(p, st);
+        case 5: return launch_narrow<5>(p, st);
+        case 6: return launch_narrow<6>(p, st);
+        case 7: return launch_narrow<7>(p, st);
+        case 8: return launch_narrow<8>(p, st);
+        case 9: return launch_narrow<9>(p, st);
+        case 10: return launch_narrow<10>(p, st);
+        case 11: return launch_narrow<11>(p, st);
+        case 12: return launch_narrow<12>(p, st);
+        default: return cudaErrorInvalidValue;
+    }
 }
 
 }  // namespace tb

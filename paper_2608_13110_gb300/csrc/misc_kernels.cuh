@@ -1,5 +1,5 @@
 // Row-0 writer, last-row reduction, amplitude finalisation and the
-// whole-sweep-in-shared-memory kernel for narrow boundaries
+// whole-sweep-on-chip kernels for narrow boundaries
 // (arXiv 2608.13110, Sec. 3.1, Algorithm 1: B <- pi[1] is the first row's
 // contraction, the loop absorbs rows 2..n, and the result is a scalar).
 #pragma once
@@ -52,12 +52,10 @@ struct FinalizeParams {
 
 struct SmallParams {
     int n, h, nb;
+    int nsm;               // SMs of the device
     const uint8_t* bits;
     const StepG* steps;
-    const int8_t* tgt;
-    const int8_t* ctl;
     const int16_t* xq;
-    const int32_t* row_end;
     int nrows;
     const float2* init_low;  // [2^h]
     const float2* init_top;  // [2 (x)][2 (bit h-1)]

@@ -808,10 +808,7 @@ int plan_build(Plan& P, int n, int d, const uint8_t* cliff, const uint8_t* tmask
     const int64_t ns = (int64_t)P.steps.size();
     L.steps = put(ns * (int64_t)sizeof(StepG));
     L.pass_steps = put((int64_t)P.pass_steps.size() * (int64_t)sizeof(StepG));
-    L.step_tgt = put(ns);
-    L.step_ctl = put(ns);
     L.step_xq = put(ns * 2);
-    L.row_end = put((int64_t)P.row_end.size() * 4);
     L.init_low = put((int64_t)P.init_low.size() * 8);
     L.init_mid = put((int64_t)P.init_mid.size() * 8);
     L.init_top = put((int64_t)P.init_top.size() * 8);
@@ -830,10 +827,7 @@ int plan_build(Plan& P, int n, int d, const uint8_t* cliff, const uint8_t* tmask
     };
     cp(L.steps, P.steps.data(), P.steps.size() * sizeof(StepG));
     cp(L.pass_steps, P.pass_steps.data(), P.pass_steps.size() * sizeof(StepG));
-    cp(L.step_tgt, P.step_tgt.data(), P.step_tgt.size());
-    cp(L.step_ctl, P.step_ctl.data(), P.step_ctl.size());
     cp(L.step_xq, P.step_xq.data(), P.step_xq.size() * 2);
-    cp(L.row_end, P.row_end.data(), P.row_end.size() * 4);
     cp(L.init_low, P.init_low.data(), P.init_low.size() * 8);
     cp(L.init_mid, P.init_mid.data(), P.init_mid.size() * 8);
     cp(L.init_top, P.init_top.data(), P.init_top.size() * 8);

@@ -23,7 +23,6 @@ constexpr int MAX_WINDOW_HIGH = TILE_BITS - 3;  // other windows keep >= 8 conse
 // Boundaries of width <= SMALL_H_MAX live in one CTA's shared memory for the
 // whole sweep (one CTA per bitstring).
 constexpr int SMALL_H_MAX = 12;
-constexpr int SMALL_THREADS = 256;
 constexpr int MAX_H = 35;        // widest boundary the device path evaluates (2^35 complex64 = 256 GiB)
 // Widest open plan whose join runs out of place into a second boundary-size
 // buffer (tensor cores, k >= JOIN_TC_MIN_K); wider open plans, and open plans
@@ -221,10 +220,7 @@ constexpr int JOIN_SEG_CHUNKS = 4;
 struct TableLayout {
     int64_t steps;     // StepG[n_steps]
     int64_t pass_steps;  // StepG[]: the steps of every pass as its kernel runs them
-    int64_t step_tgt;  // int8 target bit per step
-    int64_t step_ctl;  // int8 control bit per step (-1: none)
     int64_t step_xq;   // int16 qubit of the bitstring dependence (-1: none)
-    int64_t row_end;   // int32 index one past the last step of each absorbed row
     int64_t init_low;  // float2[2^k]          row 0: low-bit product
     int64_t init_mid;  // float2[2][2^m]       row 0: middle factor by bit k-1
     int64_t init_top;  // float2[2][2][2^top]  row 0: [x][bit k+m-1][top bits]
