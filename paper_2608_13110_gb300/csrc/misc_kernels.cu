@@ -99,6 +99,8 @@ __global__ void __launch_bounds__(REDUCE_THREADS) reduce_kernel(const ReducePara
     __shared__ double2 red[REDUCE_THREADS / 32];
     const int nk = 1 << p.k;
     for (int i = threadIdx.x; i < 2 * nk; i += blockDim.x) slow[i] = p.low[i];
+    grid_release();
+    grid_wait();
     __syncthreads();
     const int b = blockIdx.x / p.blocks_per_b;
     const int j = blockIdx.x - b * p.blocks_per_b;
@@ -146,12 +148,12 @@ cudaError_t launch_reduce(const ReduceParams& p, cudaStream_t st) {
     const int smem = (2 << p.k) * (int)sizeof(float2);
     cudaError_t e = cudaFuncSetAttribute(reduce_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
-    reduce_kernel<<<p.nbatch * p.blocks_per_b, REDUCE_THREADS, smem, st>>>(p);
-    return cudaGetLastError();
+    return launch_after(reduce_kernel, p.nbatch * p.blocks_per_b, REDUCE_THREADS, smem, st, p);
 }
 
 // psi_b = (sum of its partials) * 2^-(sum of its rescaling exponents).
 __global__ void finalize_kernel(const FinalizeParams p) {
+    grid_wait();
     const int b = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     const int l = threadIdx.x & 31;
     if (b >= p.nbatch) return;
@@ -208,8 +210,7 @@ cudaError_t launch_log_xeb(const double2* amp, int64_t nb, int n, double* out, c
 
 cudaError_t launch_finalize(const FinalizeParams& p, cudaStream_t st) {
     const int warps = 4;
-    finalize_kernel<<<(p.nbatch + warps - 1) / warps, 32 * warps, 0, st>>>(p);
-    return cudaGetLastError();
+    return launch_after(finalize_kernel, (p.nbatch + warps - 1) / warps, 32 * warps, 0, st, p);
 }
 
 // ---------------------------------------------------------------------------

@@ -641,7 +641,7 @@ __global__ void __launch_bounds__(PASS_THREADS, PASS_CTAS_PER_SM)
 
     // The producer warp (the first of the last warpgroup) works on tile
     // coordinates together; its lane 0 sets the barriers up and issues every
-    // copy. The first loads start before the coefficients are staged.
+    // copy. The first loads do not wait for the coefficients.
     if ((tid >> 5) == PASS_CONSUMERS / 32) {
         if (lane == 0) {
             asm volatile("prefetch.tensormap [%0];\n" ::"l"(reinterpret_cast<uint64_t>(&tmap)) : "memory");
@@ -653,6 +653,7 @@ __global__ void __launch_bounds__(PASS_THREADS, PASS_CTAS_PER_SM)
             asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
             asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
         }
+        grid_wait();
         if (!p.selftest)
             for (int k = 0; k < ntl && k < PASS_STAGES; ++k) {
                 tile_coords<SH>(p, first + (int64_t)k * gridDim.x, col, lane, t3[k], t4[k]);
@@ -662,7 +663,17 @@ __global__ void __launch_bounds__(PASS_THREADS, PASS_CTAS_PER_SM)
                 }
             }
     }
+    // One tile per CTA: the next pass's CTAs start on free SMs at once. With more
+    // tiles a CTA of the next pass would only hold the SM that another CTA of
+    // this pass leaves (or that another stream's work could use), so the release
+    // waits for the end. Measured (us, none / at the end / at once): n=33, d=35,
+    // one bitstring 459 / 420 / 406; n=61, d=32, 200 bitstrings 4461 / 4393 /
+    // 4413; n=28, d=42, 16 bitstrings 6643 / 6680 / 6906; plain launches 525,
+    // 4619, 6796.
+    const bool one_tile = p.ntiles <= gridDim.x;
+    if (one_tile) grid_release();
     stage_coefficients<SH>(p.steps, sc, tid);
+    grid_wait();  // every thread: the boundary and the rescaling state are the predecessor's
     __syncthreads();
 
     static_assert(PASS_THREADS - PASS_CONSUMERS == 128, "one producer warpgroup");
@@ -757,6 +768,7 @@ __global__ void __launch_bounds__(PASS_THREADS, PASS_CTAS_PER_SM)
         if (++s == PASS_STAGES) { s = 0; ph ^= 1u; }
     }
     if (cur_b >= 0) flush_max(runmax, p.maxs + cur_b * p.sstride + p.slot + 1);
+    if (!one_tile) grid_release();
 }
 
 // Launchers, one translation unit per pass type (pass_t<type>.cu).
@@ -777,8 +789,7 @@ cudaError_t launch_one(const PassParams& p, const CUtensorMap& m, int grid, cuda
         static_assert(smem <= 227 * 1024, "pass kernel shared memory");
         cudaError_t e = cudaFuncSetAttribute(pass_kernel<TYPE, M>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         if (e != cudaSuccess) return e;
-        pass_kernel<TYPE, M><<<grid, PASS_THREADS, smem, st>>>(p, m);
-        return cudaGetLastError();
+        return launch_after(pass_kernel<TYPE, M>, grid, PASS_THREADS, smem, st, p, m);
     }
 }
 

@@ -244,6 +244,34 @@ struct ScaleLayout {
     int64_t bytes_per_b;  // maxs (uint32) then exps (int32), padded
 };
 
+#ifdef __CUDACC__
+// The kernels of one sweep follow one another on a stream and each needs all of
+// its predecessor's boundary, but not to set itself up: a kernel launched with
+// launch_after may start while its predecessor's last CTAs still run, prepares
+// what does not depend on it (barriers, coefficients, tables) and then waits in
+// grid_wait for the predecessor's completion and its writes. grid_release in the
+// predecessor allows that start as soon as every one of its CTAs is running, so
+// no CTA waits for one that has no SM.
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
+__device__ __forceinline__ void grid_release() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
+
+template <class... P, class... A>
+cudaError_t launch_after(void (*kernel)(P...), unsigned grid, unsigned threads, size_t smem, cudaStream_t st,
+                         const A&... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr = {};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+#endif
+
 constexpr int64_t align_up(int64_t x, int64_t a) { return (x + a - 1) / a * a; }
 
 }  // namespace tb
