@@ -26,8 +26,9 @@ struct ReduceParams {
     const float2* B;
     int64_t b_stride;
     int h, k, m, top, n;
-    int chunk_shift;     // h - k
-    int blocks_per_b;
+    int chunk_shift;     // log2(chunks visited per batch element) = h - k - skip.n
+    TileSkip skip;       // which chunks are visited (the others are zero)
+    int blocks_per_b;    // partial sums per batch element
     int nbatch;
     const uint8_t* bits;
     const float2* low;   // [2^k][2] column vectors
@@ -74,7 +75,7 @@ constexpr int REDUCE_THREADS = 256;
 constexpr int MAX_RED_BLOCKS = 1024;
 
 cudaError_t launch_init(const InitParams& p, int grid, cudaStream_t st);
-cudaError_t launch_reduce(const ReduceParams& p, cudaStream_t st);
+cudaError_t launch_reduce(const ReduceParams& p, int nsm, cudaStream_t st);
 cudaError_t launch_finalize(const FinalizeParams& p, cudaStream_t st);
 // log-XEB estimator of nb device amplitudes (FP64, one CTA, fixed order).
 cudaError_t launch_log_xeb(const double2* amp, int64_t nb, int n, double* out, cudaStream_t st);

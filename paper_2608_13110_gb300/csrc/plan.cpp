@@ -431,6 +431,11 @@ static void tile_skips(Plan& P, Support s) {
         if (finite) advance(d.step0);
         d.skip = s.skip(outside, h);
     }
+    outside.clear();
+    for (int b = P.k; b < h; ++b) outside.push_back(b);
+    if ((int)outside.size() > MAX_TILE_BITS) return;
+    if (finite) advance((int)P.steps.size());
+    P.red_skip = s.skip(outside, h);
 }
 
 // Modelled time of a schedule in units of one HBM pass, a heuristic for the

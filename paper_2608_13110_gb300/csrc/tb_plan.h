@@ -52,6 +52,7 @@ struct Plan {
     int n_pass_launches() const {
         return opts.precision != TB_PRECISION_FP32 ? (int)tc_passes.size() : (int)passes.size();
     }
+    TileSkip red_skip{};  // 2^k-entry chunks the last-row reduction visits
     // row-0 and last-row tables
     int k = 0, m = 0, top = 0;
     std::vector<float2> init_low, init_mid, init_top, red_low, red_mid, red_top;

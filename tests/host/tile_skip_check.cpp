@@ -101,6 +101,11 @@ int main(int argc, char** argv) {
             if (b < p.lo || b >= p.lo + P.tc_wb) { tile.push_back(b); ++low; }
         if (!check(p.step0, tile, p.skip)) return 2;
     }
+    {  // the chunks of the last-row reduction
+        std::vector<int> low;
+        for (int b = 0; b < P.k; ++b) low.push_back(b);
+        if (!check((int)P.steps.size(), low, P.red_skip)) return 2;
+    }
     printf("visited=%.3f\n", visited / total);
     return 0;
 }
