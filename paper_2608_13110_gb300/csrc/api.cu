@@ -140,8 +140,8 @@ int num_sms() {
 // The pass kernel moves whole tiles with tensor copies. Its map views nbatch
 // consecutive boundaries of 2^h complex64 entries as FP32 elements in five
 // dimensions whose box is one tile (see the slot layout in pass_kernel.cuh):
-//   window at bit 0: [address bits 0..3 (32 floats)][bits 5..12][bit 4]
-//                    [tile index with batch][1];
+//   window at bit 0: [address bits 0..3 (32 floats)][bits 5..CB-1][bit 4]
+//                    [chunk index with batch][1] (box = one chunk of 2^CB);
 //   other windows, C = 13 - M >= 4 low bits, window at bits lo..lo+M-1:
 //     C = 4: [bits 0..3][window bits 0..7][window bit 8][bits 4..lo-1][rest];
 //     C > 4: [bits 0..3][bits 4..C-1][window][bits C..lo-1][rest],
@@ -174,10 +174,10 @@ int encode_pass_map(CUtensorMap* m, const PassDesc& d, const float2* B, int h, i
     const cuuint32_t estr[5] = {1, 1, 1, 1, 1};
     const cuuint64_t E = 8;  // bytes per entry
     if (is_bottom_pass(d.type)) {
-        const cuuint64_t tiles = (cuuint64_t)nbatch << (h - TILE_BITS);
-        dim[0] = 32; dim[1] = 256; dim[2] = 2; dim[3] = tiles; dim[4] = 1;
-        stride[0] = 32 * E; stride[1] = 16 * E; stride[2] = (cuuint64_t)TILE * E; stride[3] = (cuuint64_t)TILE * E;
-        box[0] = 32; box[1] = 256; box[2] = 2; box[3] = 1; box[4] = 1;
+        const int CB = bot_chunk_bits(d.M);
+        dim[0] = 32; dim[1] = (cuuint64_t)1 << (CB - 5); dim[2] = 2; dim[3] = (cuuint64_t)nbatch << (h - CB); dim[4] = 1;
+        stride[0] = 32 * E; stride[1] = 16 * E; stride[2] = E << CB; stride[3] = E << CB;
+        box[0] = 32; box[1] = (cuuint32_t)1 << (CB - 5); box[2] = 2; box[3] = 1; box[4] = 1;
     } else {
         const int M = d.M, lo = d.lo, C = TILE_BITS - M;
         if (C < 3 || lo < C || lo + M > h) return fail(TB_EINVAL, "pass window outside the tensor-copy layout");

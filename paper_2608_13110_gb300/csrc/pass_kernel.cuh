@@ -92,6 +92,8 @@ struct Shape {
     static constexpr int BLK = pass_blk(TYPE, M);         // the turn's 4x4 block (-1: none)
     static constexpr int NB = 2 * NS + (XM >= 0 ? 2 : 0);  // coefficient blocks
     static constexpr int C = BOT ? 0 : TILE_BITS - M;  // tile bit of window bit 0
+    static constexpr int CB = BOT ? bot_chunk_bits(M) : 0;   // chunks of a tile at bit 0
+    static constexpr int NCH = BOT ? 1 << (TILE_BITS - CB) : 1;  // copies per tile
     static constexpr int LAY = BOT ? LAY_BOT : (C == 3 ? LAY_LOW3 : LAY_HIGH);
     static constexpr int REG0 = BOT ? 5 : 8;            // tile bit of register bit 0
     static constexpr int regpos(int t) { return (t >= REG0 && t < REG0 + REG_BITS) ? t - REG0 : -1; }
@@ -137,7 +139,8 @@ __device__ __forceinline__ uint32_t thread_base(uint32_t tid) {
 //   * windows above bit 0: identity order. Lanes 0..3 hold tile bits 0, 4,
 //     5, 6 and the warp index bits 1..3, so the swizzled bits 0..3 are
 //     t0, t1^t4, t2^t5, t3^t6: a bijection of the lane bits.
-//   * windows at bit 0: tile bits 0..3, then 5..12, then 4. Lanes 0..3 hold
+//   * windows at bit 0, per chunk of 2^CB entries: tile bits 0..3, then
+//     5..CB-1, then 4; then the chunk (tile bits CB..12). Lanes 0..3 hold
 //     tile bits 0..3 and registers bits 5..7, so the swizzled bits are
 //     t0, t1^t5, t2^t6, t3^t7: again a bijection of the lane bits.
 //   * 10-bit windows above bit 0 (LAY_LOW3): identity order in rows of 64
@@ -153,16 +156,18 @@ __host__ __device__ constexpr uint32_t swz128(uint32_t s) { return s ^ (((s >> 4
 // 64-byte swizzle (rows of 64 bytes, LAY_LOW3): slot bits 1..2 ^= 4..5.
 __host__ __device__ constexpr uint32_t swz64(uint32_t s) { return s ^ (((s >> 4) & 3u) << 1); }
 
-template <int LAY>
+template <int LAY, int CB>
 __host__ __device__ constexpr uint32_t slot_of(uint32_t idx) {
     if (LAY == LAY_LOW3) return swz64(idx);
-    constexpr bool BOT = LAY == LAY_BOT;
-    return swz128(BOT ? ((idx & 15u) | (((idx >> 5) & 255u) << 4) | (((idx >> 4) & 1u) << 12)) : idx);
+    constexpr uint32_t MID = LAY == LAY_BOT ? (1u << (CB - 5)) - 1u : 0u;  // bits 5..CB-1
+    return swz128(LAY == LAY_BOT ? ((idx & 15u) | (((idx >> 5) & MID) << 4) | (((idx >> 4) & 1u) << (CB - 1)) |
+                                    ((idx >> CB) << CB))
+                                 : idx);
 }
 
-template <int LAY, uint32_t J>
+template <int LAY, int CB, uint32_t J>
 struct SlotC {
-    static constexpr uint32_t v = slot_of<LAY>(J);
+    static constexpr uint32_t v = slot_of<LAY, CB>(J);
 };
 
 // ---------------------------------------------------------------------------
@@ -433,23 +438,23 @@ __device__ __forceinline__ void stage_coefficients(const StepG* steps, float2* s
 
 // Registers <-> shared stage: entry j of a thread sits at tile coordinate
 // thread_base | j << REG0, i.e. slot base ^ SlotC<j << REG0>.
-template <int LAY, int REG0, int J>
+template <int LAY, int CB, int REG0, int J>
 __device__ __forceinline__ void smem_read_j(float2 (&P)[16], float2 (&Q)[16], const float2* tile, uint32_t sb) {
     if constexpr (J < 32) {
-        const float2 e = tile[sb ^ SlotC<LAY, ((uint32_t)J << REG0)>::v];
+        const float2 e = tile[sb ^ SlotC<LAY, CB, ((uint32_t)J << REG0)>::v];
         if constexpr (J < 16) { P[J].x = e.x; Q[J].x = e.y; }
         else                  { P[J - 16].y = e.x; Q[J - 16].y = e.y; }
-        smem_read_j<LAY, REG0, J + 1>(P, Q, tile, sb);
+        smem_read_j<LAY, CB, REG0, J + 1>(P, Q, tile, sb);
     }
 }
 
-template <int LAY, int REG0, int J>
+template <int LAY, int CB, int REG0, int J>
 __device__ __forceinline__ void smem_write_j(const float2 (&P)[16], const float2 (&Q)[16], float2* tile,
                                              uint32_t sb) {
     if constexpr (J < 32) {
-        tile[sb ^ SlotC<LAY, ((uint32_t)J << REG0)>::v] =
+        tile[sb ^ SlotC<LAY, CB, ((uint32_t)J << REG0)>::v] =
             J < 16 ? make_float2(P[J & 15].x, Q[J & 15].x) : make_float2(P[J & 15].y, Q[J & 15].y);
-        smem_write_j<LAY, REG0, J + 1>(P, Q, tile, sb);
+        smem_write_j<LAY, CB, REG0, J + 1>(P, Q, tile, sb);
     }
 }
 
@@ -589,18 +594,21 @@ __device__ __forceinline__ void tma_wait_all() { asm volatile("cp.async.bulk.wai
 
 // Tensor-map coordinates (dimensions 3 and 4) of visited tile gt (the whole
 // producer warp, col = this lane's column of the tile map). Windows at bit 0:
-// dimension 3 is the tile index with the batch element. Other windows:
+// lane j < NCH gets dimension 3 = the index of the tile's chunk j, with the
+// batch element; chunk = the XOR of the columns of j's bits. Other windows:
 // dimension 3 = the address bits between the low bits and the window,
 // dimension 4 = the bits above the window and the batch element.
 template <class SH>
-__device__ __forceinline__ void tile_coords(const PassParams& p, int64_t gt, uint32_t col, uint32_t lane, int& c3,
-                                            int& c4) {
+__device__ __forceinline__ void tile_coords(const PassParams& p, int64_t gt, uint32_t col, uint32_t lane,
+                                            uint32_t chunk, int& c3, int& c4) {
     const int64_t b = gt >> p.tile_shift;
-    const int64_t t = tile_of_warp(p.skip.base, col, lane, (uint32_t)(gt & (((int64_t)1 << p.tile_shift) - 1)));
+    const uint32_t u = (uint32_t)(gt & (((int64_t)1 << p.tile_shift) - 1));
     if constexpr (SH::BOT) {
-        c3 = (int)((b << (p.h - TILE_BITS)) + t);
+        const int64_t t = tile_of_warp(p.skip.base, col, lane, u << (TILE_BITS - SH::CB)) ^ chunk;
+        c3 = (int)((b << (p.h - SH::CB)) + t);
         c4 = 0;
     } else {
+        const int64_t t = tile_of_warp(p.skip.base, col, lane, u);
         const int nl = p.lo - SH::C;
         c3 = (int)(t & (((int64_t)1 << nl) - 1));
         c4 = (int)((b << (p.h - p.lo - SH::M)) + (t >> nl));
@@ -637,6 +645,17 @@ __global__ void __launch_bounds__(PASS_THREADS, PASS_CTAS_PER_SM)
     const uint32_t tries = p.selftest ? PASS_SELFTEST_TRIES : PASS_WAIT_TRIES;
     const uint32_t lane = tid & 31u;
     const uint32_t col = tile_col(p.skip, lane);
+    // copies of a tile: one per chunk at bit 0, issued by as many lanes
+    constexpr uint32_t PART = TILE_BYTES / SH::NCH;
+    const bool mover = lane < (uint32_t)SH::NCH;
+    uint32_t chunk = 0;
+    if constexpr (SH::BOT) {
+#pragma unroll
+        for (int i = 0; i < TILE_BITS - SH::CB; ++i) {
+            const uint32_t ci = __shfl_sync(0xffffffffu, col, i);
+            if (lane >> i & 1u) chunk ^= ci;
+        }
+    }
     int t3[PASS_STAGES], t4[PASS_STAGES];  // producer: coordinates of the tile in each stage
 
     // The producer warp (the first of the last warpgroup) works on tile
@@ -656,11 +675,10 @@ __global__ void __launch_bounds__(PASS_THREADS, PASS_CTAS_PER_SM)
         grid_wait();
         if (!p.selftest)
             for (int k = 0; k < ntl && k < PASS_STAGES; ++k) {
-                tile_coords<SH>(p, first + (int64_t)k * gridDim.x, col, lane, t3[k], t4[k]);
-                if (lane == 0) {
-                    pbar_expect_tx(full0 + 8 * k, TILE_BYTES);
-                    tma_load_tile(stage0 + (uint32_t)k * TILE_BYTES, &tmap, t3[k], t4[k], full0 + 8 * k);
-                }
+                tile_coords<SH>(p, first + (int64_t)k * gridDim.x, col, lane, chunk, t3[k], t4[k]);
+                if (lane == 0) pbar_expect_tx(full0 + 8 * k, TILE_BYTES);
+                __syncwarp();
+                if (mover) tma_load_tile(stage0 + (uint32_t)k * TILE_BYTES + lane * PART, &tmap, t3[k], t4[k], full0 + 8 * k);
             }
     }
     // One tile per CTA: the next pass's CTAs start on free SMs at once. With more
@@ -690,29 +708,28 @@ __global__ void __launch_bounds__(PASS_THREADS, PASS_CTAS_PER_SM)
         uint32_t ph = 0;
         for (int64_t k = 0; k < ntl; ++k) {
             int n3 = 0, n4 = 0;  // the stage's next tile, worked out while the consumers are busy
-            if (k + PASS_STAGES < ntl) tile_coords<SH>(p, first + (k + PASS_STAGES) * gridDim.x, col, lane, n3, n4);
+            if (k + PASS_STAGES < ntl) tile_coords<SH>(p, first + (k + PASS_STAGES) * gridDim.x, col, lane, chunk, n3, n4);
             const bool gave_up = !pbar_wait(done0 + 8 * s, ph, tries);
             if (__any_sync(0xffffffffu, gave_up)) {
                 if (lane == 0 && atomicExch(s_abort, 1) == 0) atomicAdd(p.fault, 1);
                 break;
             }
-            if (lane == 0) {
-                tma_store_tile(&tmap, t3[s], t4[s], stage0 + (uint32_t)s * TILE_BYTES);
-                if (k + PASS_STAGES < ntl) {
-                    tma_wait_read_all();  // the store has read the stage
-                    pbar_expect_tx(full0 + 8 * s, TILE_BYTES);
-                    tma_load_tile(stage0 + (uint32_t)s * TILE_BYTES, &tmap, n3, n4, full0 + 8 * s);
-                    last_load[s] = k + PASS_STAGES;
-                    t3[s] = n3;
-                    t4[s] = n4;
-                }
+            if (mover) tma_store_tile(&tmap, t3[s], t4[s], stage0 + (uint32_t)s * TILE_BYTES + lane * PART);
+            if (k + PASS_STAGES < ntl) {
+                if (mover) tma_wait_read_all();  // the stores have read the stage
+                if (lane == 0) pbar_expect_tx(full0 + 8 * s, TILE_BYTES);
+                __syncwarp();
+                if (mover) tma_load_tile(stage0 + (uint32_t)s * TILE_BYTES + lane * PART, &tmap, n3, n4, full0 + 8 * s);
+                last_load[s] = k + PASS_STAGES;
+                t3[s] = n3;
+                t4[s] = n4;
             }
             __syncwarp();
             if (++s == PASS_STAGES) { s = 0; ph ^= 1u; }
         }
-        if (lane != 0) return;
-        tma_wait_all();
-        if (*(volatile int*)s_abort) {
+        if (mover) tma_wait_all();
+        __syncwarp();
+        if (lane == 0 && *(volatile int*)s_abort) {
             // loads still in flight must land before the CTA's shared memory goes
             for (int st = 0; st < PASS_STAGES; ++st)
                 if (last_load[st] >= 0)
@@ -729,7 +746,7 @@ __global__ void __launch_bounds__(PASS_THREADS, PASS_CTAS_PER_SM)
     float scale = 1.0f;
     uint32_t xmask = 0;
     const int64_t tmask = ((int64_t)1 << p.tile_shift) - 1;
-    const uint32_t sb = slot_of<SH::LAY>(thread_base<SH::LAY>(tid));
+    const uint32_t sb = slot_of<SH::LAY, SH::CB>(thread_base<SH::LAY>(tid));
     int s = 0;
     uint32_t ph = 0;
     for (int64_t k = 0; k < ntl; ++k) {
@@ -756,12 +773,12 @@ __global__ void __launch_bounds__(PASS_THREADS, PASS_CTAS_PER_SM)
 
         float2* tile = stages + s * TILE;
         float2 P[16], Q[16];
-        smem_read_j<SH::LAY, SH::REG0, 0>(P, Q, tile, sb);
+        smem_read_j<SH::LAY, SH::CB, SH::REG0, 0>(P, Q, tile, sb);
         run_steps<SH, 0>(P, Q, sc, xmask, scale, tid);
 #pragma unroll
         for (int j = 0; j < 16; ++j)
             runmax = fmaxf(runmax, fmaxf(fmaxf(fabsf(P[j].x), fabsf(P[j].y)), fmaxf(fabsf(Q[j].x), fabsf(Q[j].y))));
-        smem_write_j<SH::LAY, SH::REG0, 0>(P, Q, tile, sb);
+        smem_write_j<SH::LAY, SH::CB, SH::REG0, 0>(P, Q, tile, sb);
         asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");  // visible to the tensor store
         __syncwarp();
         if ((tid & 31u) == 0) pbar_arrive(done0 + 8 * s);

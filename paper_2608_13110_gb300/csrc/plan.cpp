@@ -354,7 +354,8 @@ public:
 
     // The tiles a pass visits: outside[i] is the address bit of tile-index bit
     // i, in ascending order.
-    TileSkip skip(const std::vector<int>& outside, int h) const {
+    // At most max_n equations are used.
+    TileSkip skip(const std::vector<int>& outside, int h, int max_n = MAX_TILE_BITS) const {
         Support s = *this;
         uint64_t out = 0;
         for (int b : outside) out |= (uint64_t)1 << b;
@@ -369,6 +370,7 @@ public:
                 if (m >> outside[i] & 1) r |= (uint32_t)1 << i;
             return r;
         };
+        if ((int)s.eq_.size() > max_n) s.eq_.resize(max_n);
         // reduced equations: each pivot bit is determined by bits that are no pivots
         uint32_t pivots = 0;
         for (const Eq& e : s.eq_) {
@@ -414,13 +416,15 @@ static void tile_skips(Plan& P, Support s) {
     if (!finite) s = Support();
     std::vector<int> outside;
     for (PassDesc& d : P.passes) {
-        const int C = is_bottom(d.type) ? TILE_BITS : TILE_BITS - d.M;  // low address bits of a tile
+        // low address bits of a tile, or of a chunk at bit 0 (a tile there needs
+        // 2^(TILE_BITS - C) visited chunks)
+        const int C = is_bottom(d.type) ? bot_chunk_bits(d.M) : TILE_BITS - d.M;
         outside.clear();
         for (int b = C; b < h; ++b)
             if (is_bottom(d.type) || b < d.lo || b >= d.lo + d.M) outside.push_back(b);
         if ((int)outside.size() > MAX_TILE_BITS) continue;  // wider than the device evaluates
         if (finite) advance(d.step0);
-        d.skip = s.skip(outside, h);
+        d.skip = s.skip(outside, h, is_bottom(d.type) ? h - TILE_BITS : MAX_TILE_BITS);
     }
     for (TcPass& d : P.tc_passes) {
         outside.clear();

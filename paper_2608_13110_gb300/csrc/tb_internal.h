@@ -114,13 +114,14 @@ static_assert(sizeof(StepG) == 16 * sizeof(float2), "StepG entries are read as r
 // The other tiles are zero before the pass and stay zero, and every boundary
 // buffer holds those zeros explicitly (the row-0 writer writes all entries),
 // so leaving them alone changes no value. A pass's tile index t numbers the
-// address bits outside its tile in ascending order; n of its bits are
+// address bits outside its tile in ascending order (a window at bit 0: outside
+// its chunks of 2^CB consecutive entries, see bot_chunk_bits); n of its bits are
 // determined by the others, and the visited tiles u = 0 .. 2^(bits-n)-1 are
 // t = tile_of(u), an affine map over GF(2): base XOR the columns of u's set
 // bits. A warp evaluates it with one column per lane and one XOR reduction
 // (the loop form below costs one thread 2 us per pass when the code and the
 // arguments are cold: 0.58 against 0.52 ms for a whole width-18 amplitude).
-constexpr int MAX_TILE_BITS = 24;
+constexpr int MAX_TILE_BITS = 28;
 struct TileSkip {
     int n;
     uint32_t base;
@@ -143,6 +144,15 @@ __device__ __forceinline__ uint32_t tile_of_warp(uint32_t base, uint32_t col, ui
     return base ^ __reduce_xor_sync(0xffffffffu, (u >> lane & 1u) ? col : 0u);
 }
 #endif
+
+// A tile of a pass at address bit 0 is 2^(TILE_BITS-CB) chunks of 2^CB
+// consecutive entries: the window and, for windows of less than 8 bits, the bits
+// up to 7 (the shared-memory swizzle spans tile bits 5..7). Which chunks share a
+// tile is free, so a tile takes consecutive visited ones, and the bits between
+// the window and the tile size count as outside bits for the zeros too: with
+// random Clifford + T gates 0.75 (CB = 8) to 0.84 (CB = 10) of the chunks that
+// tiles of 2^13 consecutive entries would visit.
+__host__ __device__ constexpr int bot_chunk_bits(int M) { return M < 8 ? 8 : M; }
 
 // Host-side description of one pass (launch arguments).
 struct PassDesc {
