@@ -142,9 +142,9 @@ int num_sms() {
 // dimensions whose box is one tile (see the slot layout in pass_kernel.cuh):
 //   window at bit 0: [address bits 0..3 (32 floats)][bits 5..CB-1][bit 4]
 //                    [chunk index with batch][1] (box = one chunk of 2^CB);
-//   other windows, C = 13 - M >= 4 low bits, window at bits lo..lo+M-1:
-//     C = 4: [bits 0..3][window bits 0..7][window bit 8][bits 4..lo-1][rest];
-//     C > 4: [bits 0..3][bits 4..C-1][window][bits C..lo-1][rest],
+//   other windows, M <= 9 bits lo..lo+M-1 (box = the rows of one chunk):
+//     [bits 0..3][window, at most 8 bits][window bit 8][bits 4..lo-1][rest],
+//   10 bits: [bits 0..2][window bits 0..7][window bits 8, 9][bits 3..lo-1][rest],
 //   rest = the bits above the window and the batch element.
 using EncodeTiledFn = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
                                    const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
@@ -163,8 +163,6 @@ EncodeTiledFn encode_tiled_fn() {
     return fn;
 }
 
-bool is_bottom_pass(int type) { return type == P_BOT || type == P_BOT_START || type == P_BOT_END; }
-
 int encode_pass_map(CUtensorMap* m, const PassDesc& d, const float2* B, int h, int64_t nbatch) {
     EncodeTiledFn enc = encode_tiled_fn();
     if (!enc) return fail(TB_ECUDA, "cuTensorMapEncodeTiled is not available from the driver");
@@ -173,34 +171,24 @@ int encode_pass_map(CUtensorMap* m, const PassDesc& d, const float2* B, int h, i
     cuuint32_t box[5];
     const cuuint32_t estr[5] = {1, 1, 1, 1, 1};
     const cuuint64_t E = 8;  // bytes per entry
-    if (is_bottom_pass(d.type)) {
+    if (bottom_type(d.type)) {
         const int CB = bot_chunk_bits(d.M);
         dim[0] = 32; dim[1] = (cuuint64_t)1 << (CB - 5); dim[2] = 2; dim[3] = (cuuint64_t)nbatch << (h - CB); dim[4] = 1;
         stride[0] = 32 * E; stride[1] = 16 * E; stride[2] = E << CB; stride[3] = E << CB;
         box[0] = 32; box[1] = (cuuint32_t)1 << (CB - 5); box[2] = 2; box[3] = 1; box[4] = 1;
     } else {
-        const int M = d.M, lo = d.lo, C = TILE_BITS - M;
-        if (C < 3 || lo < C || lo + M > h) return fail(TB_EINVAL, "pass window outside the tensor-copy layout");
-        const cuuint64_t rest = (cuuint64_t)nbatch << (h - lo - M);
-        dim[0] = 32;
-        stride[2] = (E << C);  // bits C..lo-1
-        stride[3] = (E << (lo + M));
+        const int M = d.M, lo = d.lo, C = high_low_bits(M), W1 = M < 8 ? M : 8;
+        if (M < MIN_WINDOW || C < 3 || lo < C || lo + M > h) return fail(TB_EINVAL, "pass window outside the tensor-copy layout");
+        // 2^C entries per row (64 or 128 bytes), the window as 2^W1 x 2^(M-W1)
+        dim[0] = (cuuint64_t)2 << C; dim[1] = (cuuint64_t)1 << W1; dim[2] = (cuuint64_t)1 << (M - W1);
         dim[3] = (cuuint64_t)1 << (lo - C);
-        dim[4] = rest;
-        box[0] = 32; box[3] = 1; box[4] = 1;
-        if (C <= 4) {  // 2^C entries per row (64 or 128 bytes), the window as 256 x 2^(M-8)
-            dim[0] = (cuuint64_t)2 << C; box[0] = (cuuint32_t)2 << C;
-            dim[1] = 256; dim[2] = (cuuint64_t)1 << (M - 8);
-            stride[0] = E << lo; stride[1] = E << (lo + 8);
-            box[1] = 256; box[2] = (cuuint32_t)1 << (M - 8);
-        } else {
-            dim[1] = (cuuint64_t)1 << (C - 4); dim[2] = (cuuint64_t)1 << M;
-            stride[0] = 16 * E; stride[1] = E << lo;
-            box[1] = (cuuint32_t)1 << (C - 4); box[2] = (cuuint32_t)1 << M;
-        }
+        dim[4] = (cuuint64_t)nbatch << (h - lo - M);
+        stride[0] = E << lo; stride[1] = E << (lo + W1); stride[2] = E << C; stride[3] = E << (lo + M);
+        for (int i = 0; i < 3; ++i) box[i] = (cuuint32_t)dim[i];
+        box[3] = 1; box[4] = 1;
     }
     // rows of 64 bytes (a 10-bit window above bit 0) take the 64-byte swizzle
-    const bool row64 = !is_bottom_pass(d.type) && TILE_BITS - d.M == 3;
+    const bool row64 = !bottom_type(d.type) && TILE_BITS - d.M == 3;
     const CUresult r = enc(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 5, const_cast<float2*>(B), dim, stride, box, estr,
                            CU_TENSOR_MAP_INTERLEAVE_NONE, row64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B,
                            CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);

@@ -71,36 +71,38 @@ __device__ __forceinline__ uint32_t pass_smem_u32(const void* p) {
 }
 
 // Tile bits (13) of a pass and where a consumer thread holds them.
-//   LAY_BOT, windows at address bit 0 (tile = the 13 lowest address bits,
-//   window bits 0..M-1, M <= 10): lanes hold tile bits 0..4, registers
-//   5..9, the warp index 10..12;
-//   LAY_HIGH, other windows of M <= 9 bits (tile bits 0..C-1 = the C >= 4
-//   lowest address bits, tile bits C..12 = the window): lane bits 0..4 hold
-//   tile bits 0, 4, 5, 6, 7, registers 8..12, the warp index 1..3;
-//   LAY_LOW3, other windows of 10 bits (C = 3: tile bits 0..2 = the 3 lowest
-//   address bits, rows of 64 bytes): lanes hold tile bits 3..7, registers
-//   8..12, the warp index 0..2.
+//   LAY_BOT, windows at address bit 0 (tile bits 0..CB-1 = the lowest address
+//     bits, window bits 0..M-1; then the chunk): lanes hold tile bits 0..4,
+//     registers 5..9, the warp index 10..12;
+//   LAY_HIGH, other windows of M <= 9 bits (tile bits 0..3 = the 4 lowest
+//     address bits, 4..M+3 the window, then the chunk): registers hold the
+//     window's 5 highest bits, lanes its others and tile bit 0; the lanes that
+//     are left and the warp index hold tile bits 1..3 and the chunk
+//     (thread_base);
+//   LAY_LOW3, other windows of 10 bits (tile bits 0..2 = the 3 lowest
+//     address bits, rows of 64 bytes): lanes hold tile bits 3..7, registers
+//     8..12, the warp index 0..2.
 // Every window bit is a lane or register bit in each case.
 constexpr int LAY_BOT = 0, LAY_HIGH = 1, LAY_LOW3 = 2;
 template <int TYPE_, int M_>
 struct Shape {
     static constexpr int TYPE = TYPE_;
     static constexpr int M = M_;
-    static constexpr bool BOT = TYPE == P_BOT || TYPE == P_BOT_START || TYPE == P_BOT_END;
+    static constexpr bool BOT = bottom_type(TYPE);
     static constexpr int NS = pass_nsteps(TYPE, M);
     static constexpr int XM = pass_xm(TYPE, M);           // step with four variants (-1: none)
     static constexpr int BLK = pass_blk(TYPE, M);         // the turn's 4x4 block (-1: none)
     static constexpr int NB = 2 * NS + (XM >= 0 ? 2 : 0);  // coefficient blocks
-    static constexpr int C = BOT ? 0 : TILE_BITS - M;  // tile bit of window bit 0
-    static constexpr int CB = BOT ? bot_chunk_bits(M) : 0;   // chunks of a tile at bit 0
-    static constexpr int NCH = BOT ? 1 << (TILE_BITS - CB) : 1;  // copies per tile
+    static constexpr int C = BOT ? 0 : high_low_bits(M);  // tile bit of window bit 0
+    static constexpr int CB = BOT ? bot_chunk_bits(M) : 0;
+    static constexpr int CHL = pass_chunk_log2(TYPE, M);  // log2 of the chunks of a tile
     static constexpr int LAY = BOT ? LAY_BOT : (C == 3 ? LAY_LOW3 : LAY_HIGH);
-    static constexpr int REG0 = BOT ? 5 : 8;            // tile bit of register bit 0
+    static constexpr int REG0 = BOT ? 5 : C + M - REG_BITS;  // tile bit of register bit 0
     static constexpr int regpos(int t) { return (t >= REG0 && t < REG0 + REG_BITS) ? t - REG0 : -1; }
     static constexpr int lanepos(int t) {
         if (BOT) return t < 5 ? t : -1;
         if (LAY == LAY_LOW3) return (t >= 3 && t < 8) ? t - 3 : -1;
-        return t == 0 ? 0 : (t >= 4 && t < 8) ? t - 3 : -1;
+        return t == 0 ? 0 : (t >= 4 && t < REG0) ? t - 3 : -1;
     }
     static constexpr int tgt(int i) { return C + step_spec(TYPE, M, i).t; }
     static constexpr int ctl(int i) { return step_spec(TYPE, M, i).c < 0 ? -1 : C + step_spec(TYPE, M, i).c; }
@@ -120,13 +122,23 @@ struct Shape {
     }
 };
 
-// Tile coordinate of a consumer thread's register entry 0.
-template <int LAY>
+// Tile coordinate of a consumer thread's register entry 0. LAY_HIGH: tile bits
+// of the lanes, then of the warp index; the first four lanes (a half warp's
+// accesses) map to four different bank bits, see slot_of.
+template <class SH>
 __device__ __forceinline__ uint32_t thread_base(uint32_t tid) {
     const uint32_t lane = tid & 31u, warp = tid >> 5;
-    if (LAY == LAY_BOT) return lane | (warp << 10);
-    if (LAY == LAY_LOW3) return (lane << 3) | warp;
-    return (lane & 1u) | ((lane >> 1) << 4) | (warp << 1);
+    if constexpr (SH::LAY == LAY_BOT) return lane | (warp << 10);
+    if constexpr (SH::LAY == LAY_LOW3) return (lane << 3) | warp;
+    constexpr int BITS[5][8] = {{0, 1, 2, 3, 9, 10, 11, 12},   // M = 5
+                                {0, 4, 2, 3, 1, 10, 11, 12},   // 6
+                                {0, 4, 5, 3, 1, 2, 11, 12},    // 7
+                                {0, 4, 5, 6, 1, 2, 3, 12},     // 8
+                                {0, 4, 5, 6, 7, 1, 2, 3}};     // 9
+    uint32_t b = 0;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) b |= (tid >> i & 1u) << BITS[SH::M < 9 ? SH::M - 5 : 4][i];
+    return b;
 }
 
 // ---------------------------------------------------------------------------
@@ -136,9 +148,10 @@ __device__ __forceinline__ uint32_t thread_base(uint32_t tid) {
 // slot bits 1..3 with slot bits 4..6 (16-byte chunk index with the 128-byte
 // row index, stage 1024-byte aligned). A half warp's 8-byte accesses are free
 // of bank conflicts when its 16 slots differ in bits 0..3 after the swizzle.
-//   * windows above bit 0: identity order. Lanes 0..3 hold tile bits 0, 4,
-//     5, 6 and the warp index bits 1..3, so the swizzled bits 0..3 are
-//     t0, t1^t4, t2^t5, t3^t6: a bijection of the lane bits.
+//   * windows above bit 0: identity order, so the swizzled bits 0..3 are
+//     t0, t1^t4, t2^t5, t3^t6; lanes 0..3 hold tile bit 0 and one of each of
+//     the other three pairs, the registers and the warp index the rest: a
+//     bijection of the lane bits.
 //   * windows at bit 0, per chunk of 2^CB entries: tile bits 0..3, then
 //     5..CB-1, then 4; then the chunk (tile bits CB..12). Lanes 0..3 hold
 //     tile bits 0..3 and registers bits 5..7, so the swizzled bits are
@@ -592,10 +605,10 @@ __device__ __forceinline__ void tma_store_tile(const CUtensorMap* m, int c3, int
 __device__ __forceinline__ void tma_wait_read_all() { asm volatile("cp.async.bulk.wait_group.read 0;\n" ::: "memory"); }
 __device__ __forceinline__ void tma_wait_all() { asm volatile("cp.async.bulk.wait_group 0;\n" ::: "memory"); }
 
-// Tensor-map coordinates (dimensions 3 and 4) of visited tile gt (the whole
-// producer warp, col = this lane's column of the tile map). Windows at bit 0:
-// lane j < NCH gets dimension 3 = the index of the tile's chunk j, with the
-// batch element; chunk = the XOR of the columns of j's bits. Other windows:
+// Tensor-map coordinates (dimensions 3 and 4) of the chunk that this lane moves
+// of visited tile gt (the whole producer warp; col = this lane's column of the
+// tile map, chunk = the XOR of the columns of the lane's own bits). Windows at
+// bit 0: dimension 3 = the chunk index with the batch element. Other windows:
 // dimension 3 = the address bits between the low bits and the window,
 // dimension 4 = the bits above the window and the batch element.
 template <class SH>
@@ -603,12 +616,11 @@ __device__ __forceinline__ void tile_coords(const PassParams& p, int64_t gt, uin
                                             uint32_t chunk, int& c3, int& c4) {
     const int64_t b = gt >> p.tile_shift;
     const uint32_t u = (uint32_t)(gt & (((int64_t)1 << p.tile_shift) - 1));
+    const int64_t t = tile_of_warp(p.skip.base, col, lane, u << SH::CHL) ^ chunk;
     if constexpr (SH::BOT) {
-        const int64_t t = tile_of_warp(p.skip.base, col, lane, u << (TILE_BITS - SH::CB)) ^ chunk;
         c3 = (int)((b << (p.h - SH::CB)) + t);
         c4 = 0;
     } else {
-        const int64_t t = tile_of_warp(p.skip.base, col, lane, u);
         const int nl = p.lo - SH::C;
         c3 = (int)(t & (((int64_t)1 << nl) - 1));
         c4 = (int)((b << (p.h - p.lo - SH::M)) + (t >> nl));
@@ -645,16 +657,14 @@ __global__ void __launch_bounds__(PASS_THREADS, PASS_CTAS_PER_SM)
     const uint32_t tries = p.selftest ? PASS_SELFTEST_TRIES : PASS_WAIT_TRIES;
     const uint32_t lane = tid & 31u;
     const uint32_t col = tile_col(p.skip, lane);
-    // copies of a tile: one per chunk at bit 0, issued by as many lanes
-    constexpr uint32_t PART = TILE_BYTES / SH::NCH;
-    const bool mover = lane < (uint32_t)SH::NCH;
+    // copies of a tile: one per chunk, issued by as many lanes
+    constexpr uint32_t PART = TILE_BYTES >> SH::CHL;
+    const bool mover = lane < (1u << SH::CHL);
     uint32_t chunk = 0;
-    if constexpr (SH::BOT) {
 #pragma unroll
-        for (int i = 0; i < TILE_BITS - SH::CB; ++i) {
-            const uint32_t ci = __shfl_sync(0xffffffffu, col, i);
-            if (lane >> i & 1u) chunk ^= ci;
-        }
+    for (int i = 0; i < SH::CHL; ++i) {
+        const uint32_t ci = __shfl_sync(0xffffffffu, col, i);
+        if (lane >> i & 1u) chunk ^= ci;
     }
     int t3[PASS_STAGES], t4[PASS_STAGES];  // producer: coordinates of the tile in each stage
 
@@ -746,7 +756,7 @@ __global__ void __launch_bounds__(PASS_THREADS, PASS_CTAS_PER_SM)
     float scale = 1.0f;
     uint32_t xmask = 0;
     const int64_t tmask = ((int64_t)1 << p.tile_shift) - 1;
-    const uint32_t sb = slot_of<SH::LAY, SH::CB>(thread_base<SH::LAY>(tid));
+    const uint32_t sb = slot_of<SH::LAY, SH::CB>(thread_base<SH>(tid));
     int s = 0;
     uint32_t ph = 0;
     for (int64_t k = 0; k < ntl; ++k) {

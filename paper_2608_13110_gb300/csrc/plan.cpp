@@ -80,8 +80,6 @@ M2 clifford(int k) {
     return m2_mul(P[k % 4], R[k / 4]);
 }
 
-static bool is_bottom(int type) { return type == P_BOT || type == P_BOT_START || type == P_BOT_END; }
-
 static float2 f2(cd z) { return make_float2((float)z.real(), (float)z.imag()); }
 
 // ---------------------------------------------------------------------------
@@ -416,15 +414,14 @@ static void tile_skips(Plan& P, Support s) {
     if (!finite) s = Support();
     std::vector<int> outside;
     for (PassDesc& d : P.passes) {
-        // low address bits of a tile, or of a chunk at bit 0 (a tile there needs
-        // 2^(TILE_BITS - C) visited chunks)
-        const int C = is_bottom(d.type) ? bot_chunk_bits(d.M) : TILE_BITS - d.M;
+        const bool bottom = bottom_type(d.type);
+        const int C = bottom ? bot_chunk_bits(d.M) : high_low_bits(d.M);  // low address bits of a chunk
         outside.clear();
         for (int b = C; b < h; ++b)
-            if (is_bottom(d.type) || b < d.lo || b >= d.lo + d.M) outside.push_back(b);
+            if (bottom || b < d.lo || b >= d.lo + d.M) outside.push_back(b);
         if ((int)outside.size() > MAX_TILE_BITS) continue;  // wider than the device evaluates
         if (finite) advance(d.step0);
-        d.skip = s.skip(outside, h, is_bottom(d.type) ? h - TILE_BITS : MAX_TILE_BITS);
+        d.skip = s.skip(outside, h, h - TILE_BITS);  // at least one tile of visited chunks
     }
     for (TcPass& d : P.tc_passes) {
         outside.clear();

@@ -145,14 +145,23 @@ __device__ __forceinline__ uint32_t tile_of_warp(uint32_t base, uint32_t col, ui
 }
 #endif
 
-// A tile of a pass at address bit 0 is 2^(TILE_BITS-CB) chunks of 2^CB
-// consecutive entries: the window and, for windows of less than 8 bits, the bits
-// up to 7 (the shared-memory swizzle spans tile bits 5..7). Which chunks share a
-// tile is free, so a tile takes consecutive visited ones, and the bits between
-// the window and the tile size count as outside bits for the zeros too: with
-// random Clifford + T gates 0.75 (CB = 8) to 0.84 (CB = 10) of the chunks that
-// tiles of 2^13 consecutive entries would visit.
+// A tile is pass_chunks(type, M) chunks, each one tensor copy. At address bit 0
+// a chunk is 2^CB consecutive entries: the window and, for windows of less than
+// 8 bits, the bits up to 7 (the shared-memory swizzle spans tile bits 5..7).
+// Elsewhere it is the window's 2^M rows of 16 consecutive entries (128 bytes; 8
+// entries for M = 10). Which chunks share a tile is free, so a tile takes
+// consecutive visited ones, and every bit outside the chunks counts as an
+// outside bit for the zeros: with random Clifford + T gates 0.75 (CB = 8) to
+// 0.84 (CB = 10) of what tiles of 2^13 consecutive entries would visit at bit 0,
+// 0.84 (M = 6) and 0.89 (M = 7) of tiles with the 13 - M lowest bits elsewhere.
 __host__ __device__ constexpr int bot_chunk_bits(int M) { return M < 8 ? 8 : M; }
+__host__ __device__ constexpr int high_low_bits(int M) { return M > 9 ? TILE_BITS - M : 4; }
+__host__ __device__ constexpr bool bottom_type(int type) {
+    return type == P_BOT || type == P_BOT_START || type == P_BOT_END;
+}
+__host__ __device__ constexpr int pass_chunk_log2(int type, int M) {
+    return TILE_BITS - (bottom_type(type) ? bot_chunk_bits(M) : M + high_low_bits(M));
+}
 
 // Host-side description of one pass (launch arguments).
 struct PassDesc {

@@ -87,13 +87,13 @@ int main(int argc, char** argv) {
         return true;
     };
     for (const PassDesc& p : P.passes) {
-        const bool bottom = p.type == P_BOT || p.type == P_BOT_START || p.type == P_BOT_END;
+        const bool bottom = bottom_type(p.type);
         std::vector<int> tile;
-        for (int b = 0; b < (bottom ? bot_chunk_bits(p.M) : TILE_BITS - p.M); ++b) tile.push_back(b);
+        for (int b = 0; b < (bottom ? bot_chunk_bits(p.M) : high_low_bits(p.M)); ++b) tile.push_back(b);
         if (!bottom)
             for (int b = 0; b < p.M; ++b) tile.push_back(p.lo + b);
         if (!check(p.step0, tile, p.skip)) return 2;
-        if (bottom && h - bot_chunk_bits(p.M) - p.skip.n < TILE_BITS - bot_chunk_bits(p.M)) {
+        if (p.skip.n > h - TILE_BITS) {
             printf("pass at step %d visits less than one tile\n", p.step0);
             return 2;
         }
