@@ -181,9 +181,10 @@ __global__ void finalize_kernel(const FinalizeParams p) {
         sr += __shfl_xor_sync(0xffffffffu, sr, off);
         si += __shfl_xor_sync(0xffffffffu, si, off);
     }
+    int e = 0;  // |exponent| <= 100 per slot
+    for (int i = l; i < p.nslots; i += 32) e += p.exps[b * p.sstride + i];
+    const long long S = __reduce_add_sync(0xffffffffu, e);
     if (l == 0) {
-        long long S = 0;
-        for (int i = 0; i < p.nslots; ++i) S += p.exps[b * p.sstride + i];
         const int Si = (int)max(-1000000LL, min(1000000LL, S));
         p.out[2 * b] = scalbn(sr, -Si);
         p.out[2 * b + 1] = scalbn(si, -Si);

@@ -161,6 +161,13 @@ __global__ void __launch_bounds__(TC_THREADS, TC_CTAS_PER_SM) tc_pass_kernel(con
         *s_abort = 0;
     }
     tc_fence_before();
+    // the block and the tensor memory are ready; the boundary and the rescaling
+    // state are the predecessor's. The next pass's CTAs may follow as soon as
+    // one of these leaves its SM: two share it, so staging the next block (64 KB)
+    // overlaps the other's last tiles (n=32, d=48, 4 bitstrings, both forms:
+    // 28.6 ms with plain launches, 27.9 released at the end, 26.9 at once).
+    grid_release();
+    grid_wait();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tslot;
@@ -386,8 +393,7 @@ cudaError_t launch_kind(const TcParams& p, int grid, cudaStream_t st) {
         if (e != cudaSuccess) return e;
         attr = true;
     }
-    tc_pass_kernel<KIND><<<grid, TC_THREADS, C::SMEM_BYTES, st>>>(p);
-    return cudaGetLastError();
+    return launch_after(tc_pass_kernel<KIND>, grid, TC_THREADS, C::SMEM_BYTES, st, p);
 }
 
 }  // namespace
