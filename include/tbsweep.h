@@ -354,8 +354,9 @@ TB_API void tb_server_destroy(tb_server* server);
  * crossings. bytes[c] is the algorithmic HBM traffic of those launches: a
  * pass reads and writes every entry of the tiles it visits once (16 bytes per
  * entry; tiles that the plan knows to be exactly zero are not visited), a join
- * every boundary entry, the writer writes 8, the reduction reads 8, a late crossing reads
- * two entries and writes one (24 bytes per output entry). */
+ * likewise for the rows it visits, the writer writes 8, the reduction reads 8
+ * of what it visits, a late crossing reads two entries (one where the other is
+ * known to be zero) and writes one. */
 #define TB_PROFILE_CLASSES 7
 typedef struct {
     int64_t launches[TB_PROFILE_CLASSES];

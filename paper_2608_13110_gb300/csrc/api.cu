@@ -382,7 +382,8 @@ int run_device(const Plan& P, const uint8_t* d_bits, int64_t nb, void* d_ws, int
                         jp.out_stride = 0;
                         jp.Es = tab<uint8_t>(d_ws, L.open_Es);
                         jp.KR = 2 << k;
-                        jp.rows = c.join_slice_rows;
+                        jp.rows = jp.rows_all = c.join_slice_rows;
+                        jp.skip = identity_tiles();
                         jp.nbatch = 1;
                         jp.fault = fault;
                         const int64_t items = (jp.rows / 128) * (jp.KR / join_nt(k));
@@ -405,14 +406,16 @@ int run_device(const Plan& P, const uint8_t* d_bits, int64_t nb, void* d_ws, int
                 jp.out_stride = b_stride;
                 jp.Es = tab<uint8_t>(d_ws, L.open_Es);
                 jp.KR = 2 << k;
-                jp.rows = b_stride >> k;
+                jp.rows_all = b_stride >> k;
+                jp.rows = jp.rows_all >> P.join_skip.n;
+                jp.skip = P.join_skip;
                 jp.nbatch = nbat;
                 jp.fault = fault;
                 const int64_t items = (int64_t)nbat * (jp.rows / 128) * (jp.KR / join_nt(k));
                 CUtensorMap amap;
-                const int rc = encode_join_map(&amap, boundary, k, jp.rows * nbat);
+                const int rc = encode_join_map(&amap, boundary, k, jp.rows_all * nbat);
                 if (rc != TB_OK) return rc;
-                ProfScope ps(PC_JOIN, 16.0 * (double)nbat * (double)b_stride, st);
+                ProfScope ps(PC_JOIN, 16.0 * (double)nbat * (double)(jp.rows << k), st);
                 TB_CUDA(launch_join_tc(k, jp, amap, (int)std::min<int64_t>(items, nsm), st));
                 cur = second;
             } else {  // FP32, in place
@@ -441,7 +444,9 @@ int run_device(const Plan& P, const uint8_t* d_bits, int64_t nb, void* d_ws, int
                 lp.ops = ops + P.open_seg[i];
                 lp.nops = P.open_seg[i + 1] - P.open_seg[i];
                 lp.w = P.open_w[i];
-                ProfScope ps(PC_LATE, 24.0 * (double)nbat * (double)lp.out_entries, st);
+                lp.skip = P.late_skip[i];
+                ProfScope ps(PC_LATE, (lp.skip.both ? 24.0 : 16.0) * (double)nbat * (double)(lp.out_entries >> lp.skip.out.n),
+                             st);
                 TB_CUDA(launch_late(lp, 16 * nsm, st));
                 cur = nxt;
             }

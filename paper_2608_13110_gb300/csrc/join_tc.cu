@@ -81,7 +81,7 @@ __device__ __forceinline__ void expect_tx(uint32_t bar, uint32_t bytes) {
 
 template <int NT>
 __global__ void __launch_bounds__(JT_THREADS, 1)
-    join_tc_kernel(const JoinTcParams p, const __grid_constant__ CUtensorMap amap) {
+    join_tc_kernel(const __grid_constant__ JoinTcParams p, const __grid_constant__ CUtensorMap amap) {
     constexpr uint32_t PART = (uint32_t)NT * JOIN_KC * 4;  // one of hi / lo
     constexpr uint32_t BLK = 2 * PART;
     constexpr uint32_t ABYTES = 128 * JOIN_KC * 4;          // 128 rows x JOIN_KC floats
@@ -130,6 +130,11 @@ __global__ void __launch_bounds__(JT_THREADS, 1)
     const int nseg = (nkc + JOIN_SEG_CHUNKS - 1) / JOIN_SEG_CHUNKS;
     const int64_t nrb = p.rows / 128;  // row blocks per batch element
     const int64_t items = (int64_t)p.nbatch * nrb * ntn;
+    // first row, within all batch elements, of visited row block rbg
+    auto first_row = [&](int64_t rbg) {
+        const int64_t b = rbg / nrb;
+        return b * p.rows_all + (int64_t)tile_of_thread(p.skip, (uint32_t)(rbg - b * nrb)) * 128;
+    };
     // Chunk c of this CTA (counted over all its items) uses stage c % S for its
     // B block (shared memory) and A split (tensor memory); segment g (counted
     // over all items) accumulates in D[g % 2].
@@ -154,7 +159,7 @@ __global__ void __launch_bounds__(JT_THREADS, 1)
         bool ok = true;
         for (int64_t it = blockIdx.x; it < items && ok; it += gridDim.x) {
             const int nt = (int)(it % ntn);
-            const int arow0 = (int)((it / ntn) * 128);  // first row of the item (batch elements are contiguous)
+            const int arow0 = (int)first_row(it / ntn);  // first row of the item (batch elements are contiguous)
             for (int kc = 0; kc < nkc && ok; ++kc) {
                 const uint32_t cc = c + kc, s = stage_of(cc);
                 if (cc >= JT_STAGES) ok = mbar_wait(mdone0 + 8 * s, par_of(cc - JT_STAGES), JT_WAIT_TRIES);
@@ -228,9 +233,8 @@ __global__ void __launch_bounds__(JT_THREADS, 1)
     bool ok = true;
     for (int64_t it = blockIdx.x; it < items && ok; it += gridDim.x) {
         const int nt = (int)(it % ntn);
-        const int64_t rbg = it / ntn;
-        const int64_t b = rbg / nrb, rb = rbg - b * nrb;
-        const int64_t row = rb * 128 + tid;
+        const int64_t rbg = it / ntn, b = rbg / nrb;
+        const int64_t row = first_row(rbg) - b * p.rows_all + tid;
         float acc[NT];
 #pragma unroll
         for (int e = 0; e < NT; ++e) acc[e] = 0.0f;

@@ -32,6 +32,7 @@ struct LateParams {
     const OpenOp* ops;     // the segment after this crossing
     int nops;
     float2 w;              // the crossing's entangler factor (-1 for CZ)
+    LateSkip skip;         // rows written and read (skip.out.n == 0: every row is written)
 };
 
 struct OpenFinalParams {
@@ -53,7 +54,9 @@ struct JoinTcParams {
     int64_t out_stride;
     const uint8_t* Es;     // split real embedding of E (JOIN_KC x join_nt(k) blocks)
     int KR;                // 2^(k+1): reals per row
-    int64_t rows;          // rows per batch element, 2^(h-k) (a multiple of 128)
+    int64_t rows;          // rows visited per batch element, 2^(h-k-skip.n) (a multiple of 128)
+    int64_t rows_all;      // rows of a batch element, 2^(h-k)
+    TileSkip skip;         // which 128-row blocks are visited (the others are zero; Z is not written there)
     int nbatch;
     int* fault;            // bounded waits that gave up
 };

@@ -387,6 +387,14 @@ public:
         return k;
     }
 
+    // The equation that determines bit var from the higher bits, if any (after the
+    // lower bits have been eliminated): parity(address & *mask) ^ *value.
+    bool determined(int var, uint64_t* mask, int* value) const {
+        for (const Eq& e : eq_)
+            if (e.mask >> var & 1) { *mask = e.mask & ~((uint64_t)1 << var); *value = e.value; return true; }
+        return false;
+    }
+
 private:
     struct Eq {
         uint64_t mask;
@@ -432,11 +440,37 @@ static void tile_skips(Plan& P, Support s) {
         if (finite) advance(d.step0);
         d.skip = s.skip(outside, h);
     }
-    outside.clear();
-    for (int b = P.k; b < h; ++b) outside.push_back(b);
-    if ((int)outside.size() > MAX_TILE_BITS) return;
+    auto above = [&](int lo) {
+        outside.clear();
+        for (int b = lo; b < h; ++b) outside.push_back(b);
+        return (int)outside.size() <= MAX_TILE_BITS;
+    };
     if (finite) advance((int)P.steps.size());
-    P.red_skip = s.skip(outside, h);
+    if (!P.open_k) {
+        if (above(P.k)) P.red_skip = s.skip(outside, h);
+        return;
+    }
+    // open plan: the join mixes the k lowest bits, late crossing i sums bit k+i out
+    const int k = P.open_k;
+    P.late_skip.clear();
+    if (!above(k + 1)) s = Support();  // rows beyond the map: visit everything
+    if (above(k + 7)) P.join_skip = s.skip(outside, h);
+    for (int b = 0; b < k; ++b) s.eliminate(b);
+    for (size_t i = 0; i + 1 < P.open_seg.size(); ++i) {
+        LateSkip ls;
+        std::memset(&ls, 0, sizeof(ls));
+        uint64_t m = 0;
+        int v = 0;
+        ls.both = !s.determined(k + (int)i, &m, &v);
+        ls.mask = (uint32_t)(m >> (k + i + 1));
+        ls.fix = (uint32_t)v;
+        s.eliminate(k + (int)i);
+        // the last crossing's output is read in full (2^k entries, or twice
+        // that with an idle top bit)
+        if (above(k + (int)i + 1))
+            ls.out = i + 2 < P.open_seg.size() ? s.skip(outside, h) : Support().skip(outside, h);
+        P.late_skip.push_back(ls);
+    }
 }
 
 // Modelled time of a schedule in units of one HBM pass, a heuristic for the
@@ -799,13 +833,12 @@ int plan_build(Plan& P, int n, int d, const uint8_t* cliff, const uint8_t* tmask
         if (P.passes.empty()) { err = "no pass schedule fits these window limits"; return TB_EINVAL; }
         build_pass_steps(P);
     }
-    tile_skips(P, row0);
-
     sym_alg1(n, d, &P.width, &P.log2cost);
     if (P.open_k > 0) {
         const int rc = open_tables(P, err);
         if (rc != TB_OK) return rc;
     }
+    tile_skips(P, row0);
 
     // ---- device table image
     TableLayout& L = P.lay;

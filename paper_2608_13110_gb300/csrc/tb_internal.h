@@ -128,6 +128,12 @@ struct TileSkip {
     uint32_t col[MAX_TILE_BITS];
 };
 
+inline TileSkip identity_tiles() {
+    TileSkip k = {};
+    for (int i = 0; i < MAX_TILE_BITS; ++i) k.col[i] = (uint32_t)1 << i;
+    return k;
+}
+
 inline uint32_t tile_of(const TileSkip& k, uint32_t u) {
     uint32_t t = k.base;
     for (int i = 0; i < MAX_TILE_BITS; ++i)
@@ -136,6 +142,12 @@ inline uint32_t tile_of(const TileSkip& k, uint32_t u) {
 }
 
 #ifdef __CUDACC__
+// One thread (for code that only one lane runs).
+__device__ __forceinline__ uint32_t tile_of_thread(const TileSkip& k, uint32_t u) {
+    uint32_t t = k.base;
+    for (; u; u &= u - 1) t ^= k.col[__ffs(u) - 1];
+    return t;
+}
 // All 32 lanes, u uniform; col = this lane's column (tile_col).
 __device__ __forceinline__ uint32_t tile_col(const TileSkip& k, uint32_t lane) {
     return lane < MAX_TILE_BITS ? k.col[lane] : 0u;
@@ -162,6 +174,15 @@ __host__ __device__ constexpr bool bottom_type(int type) {
 __host__ __device__ constexpr int pass_chunk_log2(int type, int M) {
     return TILE_BITS - (bottom_type(type) ? bot_chunk_bits(M) : M + high_low_bits(M));
 }
+
+// Rows of a late crossing of an open plan: output rows visited, and which of
+// the input rows 2r', 2r'+1 may be nonzero (one: both == 0, the row whose low
+// bit is parity(r' & mask) ^ fix). The others are not read or written.
+struct LateSkip {
+    TileSkip out;
+    int both;
+    uint32_t mask, fix;
+};
 
 // Host-side description of one pass (launch arguments).
 struct PassDesc {

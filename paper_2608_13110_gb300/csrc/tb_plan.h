@@ -48,6 +48,8 @@ struct Plan {
     std::vector<OpenOp> open_ops;
     std::vector<int32_t> open_seg;
     std::vector<float2> open_w;  // entangler factor w of each late crossing (-1 for CZ)
+    TileSkip join_skip{};              // 128-row blocks the tensor-core join visits
+    std::vector<LateSkip> late_skip;   // rows each late crossing writes and reads
     int last_mid_row() const { return open_k ? n - open_k - 1 : n - 2; }
     int n_pass_launches() const {
         return opts.precision != TB_PRECISION_FP32 ? (int)tc_passes.size() : (int)passes.size();
