@@ -546,18 +546,60 @@ struct NarrowRun {
 };
 
 // --- h <= 7: one warp, address bits 0..4 on the lanes, the rest in registers --
-// A step on a lane bit takes the partner's entry by shuffle; each lane loads
-// the coefficient row of its own output one row ahead, so the steps wait for
-// nothing but their own chain (n = 12, d = 8, 64 bitstrings, whole host call:
-// 73 us with a CTA and a barrier per step, 54 us).
+// A step on a lane bit takes the partner's entry by shuffle. Each lane loads the
+// coefficient rows of its own outputs a group of rows ahead, with the output
+// bits already in registers, so a row waits for its own chain and not for a
+// chain of loads (width 4, 64 bitstrings: 8.1 -> 5.0 us at n = 12, 25.4 -> 12.4
+// us at n = 45; width 7, n = 45: 47 -> 32 us; a CTA and a barrier per step took
+// longer than either).
 template <int H>
 __device__ void narrow_warp(const SmallParams& p, int b) {
     constexpr int LB = H < 5 ? H : 5, R = H > 5 ? 1 << (H - 5) : 1;
+    constexpr int D = H <= 4 ? 4 : H == 5 ? 3 : H == 6 ? 2 : 1;  // rows per group
     const uint32_t lane = threadIdx.x & 31u;
     const uint8_t* xb = p.bits + (int64_t)b * p.n;
     const bool live = lane < (1u << LB);
+    uint32_t xm[4];  // output bits 0..127
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        const int q = 32 * j + (int)lane;
+        xm[j] = __ballot_sync(0xffffffffu, q < p.n && xb[q < p.n ? q : 0] != 0);
+    }
+    auto xbit = [&](int q) -> int {
+        if (q >= 128) return xb[q] ? 1 : 0;
+        const uint32_t lo = q & 32 ? xm[1] : xm[0], hi = q & 32 ? xm[3] : xm[2];
+        return (int)((q & 64 ? hi : lo) >> (q & 31) & 1u);
+    };
+    // Coefficients of a group of rows: for every target, this lane's output
+    // rows. A register target or control needs more than one: [register control
+    // or target value][2 entries]. Only the step on the highest bit depends on
+    // an output bit, its row's.
+    constexpr int NC = R > 1 ? 4 : 1;
+    float4 cur[D][H][NC], nxt[D][H][NC];
+    auto fetch = [&](int row0, float4 (&o)[D][H][NC]) {
+#pragma unroll
+        for (int r = 0; r < D; ++r) {
+            const int row = row0 + r;
+            if (row >= p.nrows) return;
+            const bool fwd = (row & 1) == 0;  // row 0 here is the circuit's row 1
+#pragma unroll
+            for (int tg = 0; tg < H; ++tg) {
+                const int st = row * H + (fwd ? tg : H - 1 - tg);
+                const float4* g = reinterpret_cast<const float4*>(p.steps[st].g[tg == H - 1 ? xbit(row + 1) : 0]);
+                const int ct = fwd ? tg - 1 : tg + 1;  // control bit (outside 0..H-1: none)
+                const bool cin = ct >= 0 && ct < H;
+#pragma unroll
+                for (int i = 0; i < NC; ++i) {
+                    const int ap = tg < LB ? (int)(lane >> tg & 1u) : (i & 1);
+                    const int c = !cin ? 0 : ct < LB ? (int)(lane >> (ct < 0 ? 0 : ct) & 1u) : (i >> 1);
+                    o[r][tg][i] = g[c * 2 + ap];
+                }
+            }
+        }
+    };
+    fetch(0, cur);
     float2 v[R];
-    const int x0 = xb[0] ? 1 : 0;
+    const int x0 = xbit(0);
 #pragma unroll
     for (int r = 0; r < R; ++r) {
         const uint32_t e = (lane & ((1u << LB) - 1u)) | ((uint32_t)r << LB);
@@ -568,38 +610,14 @@ __device__ void narrow_warp(const SmallParams& p, int b) {
         float m = 0.0f;
 #pragma unroll
         for (int r = 0; r < R; ++r) m = fmaxf(m, fmaxf(fabsf(v[r].x), fabsf(v[r].y)));
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, off));
-        const int s = rescale_exp_m(m);
+        // non-negative floats compare like their bits
+        const int s = rescale_exp_m(__uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(m))));
         const float sc = ldexpf(1.0f, s);
 #pragma unroll
         for (int r = 0; r < R; ++r) v[r] = make_float2(v[r].x * sc, v[r].y * sc);
         S += s;
     };
     rescale();
-    // coefficients of one row: for every target, this lane's output rows. A
-    // register target or control needs more than one: [register control or
-    // target value][2 entries]
-    constexpr int NC = R > 1 ? 4 : 1;
-    float4 cur[H][NC], nxt[H][NC];
-    auto fetch = [&](int row, float4 (&o)[H][NC]) {
-        if (row >= p.nrows) return;
-        const bool fwd = (row & 1) == 0;  // row 0 here is the circuit's row 1
-#pragma unroll
-        for (int tg = 0; tg < H; ++tg) {
-            const int st = row * H + (fwd ? tg : H - 1 - tg);
-            const int q = p.xq[st];
-            const float4* g = reinterpret_cast<const float4*>(p.steps[st].g[q >= 0 && xb[q] ? 1 : 0]);
-            const int ct = fwd ? tg - 1 : tg + 1;  // control bit (outside 0..H-1: none)
-            const bool cin = ct >= 0 && ct < H;
-#pragma unroll
-            for (int i = 0; i < NC; ++i) {
-                const int ap = tg < LB ? (int)(lane >> tg & 1u) : (i & 1);
-                const int c = !cin ? 0 : ct < LB ? (int)(lane >> (ct < 0 ? 0 : ct) & 1u) : (i >> 1);
-                o[tg][i] = g[c * 2 + ap];
-            }
-        }
-    };
     auto out = [](float4 g, float2 a, float2 bb) {
         return cmac2m(make_float2(g.x, g.y), a, make_float2(g.z, g.w), bb);
     };
@@ -627,23 +645,28 @@ __device__ void narrow_warp(const SmallParams& p, int b) {
             }
         }
     };
-    fetch(0, cur);
-    for (int row = 0; row < p.nrows; ++row) {
-        fetch(row + 1, nxt);
-        if ((row & 1) == 0) {
+    for (int row0 = 0; row0 < p.nrows; row0 += D) {
+        fetch(row0 + D, nxt);
 #pragma unroll
-            for (int tg = 0; tg < H; ++tg) step(tg, tg - 1, cur[tg]);
-        } else {
+        for (int r = 0; r < D; ++r) {
+            if (row0 + r >= p.nrows) break;
+            if (((row0 + r) & 1) == 0) {
 #pragma unroll
-            for (int tg = H - 1; tg >= 0; --tg) step(tg, tg + 1, cur[tg]);
+                for (int tg = 0; tg < H; ++tg) step(tg, tg - 1, cur[r][tg]);
+            } else {
+#pragma unroll
+                for (int tg = H - 1; tg >= 0; --tg) step(tg, tg + 1, cur[r][tg]);
+            }
+            rescale();
         }
-        rescale();
 #pragma unroll
-        for (int tg = 0; tg < H; ++tg)
+        for (int r = 0; r < D; ++r)
 #pragma unroll
-            for (int i = 0; i < NC; ++i) cur[tg][i] = nxt[tg][i];
+            for (int tg = 0; tg < H; ++tg)
+#pragma unroll
+                for (int i = 0; i < NC; ++i) cur[r][tg][i] = nxt[r][tg][i];
     }
-    const int xl = xb[p.n - 1] ? 1 : 0;
+    const int xl = xbit(p.n - 1);
     double ar = 0.0, ai = 0.0;
 #pragma unroll
     for (int r = 0; r < R; ++r) {
