@@ -303,86 +303,79 @@ public:
 
     // Add an equation (dependent ones are dropped).
     void add(uint64_t mask, int value) {
-        for (const Eq& e : eq_)
-            if (mask >> e.pivot & 1) { mask ^= e.mask; value ^= e.value; }
+        for (int i = 0; i < n_; ++i)
+            if (mask >> eq_[i].pivot & 1) { mask ^= eq_[i].mask; value ^= eq_[i].value; }
         if (!mask) return;
         const int pv = 63 - __builtin_clzll(mask);
-        for (Eq& e : eq_)
-            if (e.mask >> pv & 1) { e.mask ^= mask; e.value ^= value; }
-        eq_.push_back(Eq{mask, value, pv});
+        for (int i = 0; i < n_; ++i)
+            if (eq_[i].mask >> pv & 1) { eq_[i].mask ^= mask; eq_[i].value ^= value; }
+        eq_[n_++] = Eq{mask, value, pv};
     }
 
     // Project a variable out.
     void eliminate(int var) {
         int hit = -1;
-        for (size_t i = 0; i < eq_.size(); ++i)
-            if (eq_[i].mask >> var & 1) hit = (int)i;
+        for (int i = 0; i < n_; ++i)
+            if (eq_[i].mask >> var & 1) hit = i;
         if (hit < 0) return;
         const Eq h = eq_[hit];
-        std::vector<Eq> old;
-        old.swap(eq_);
-        for (size_t i = 0; i < old.size(); ++i)
-            if ((int)i != hit) {
-                const bool has = (old[i].mask >> var & 1) != 0;
-                add(has ? old[i].mask ^ h.mask : old[i].mask, has ? old[i].value ^ h.value : old[i].value);
-            }
+        eq_[hit] = eq_[--n_];
+        bool again = false;  // an equation that took h in may have lost its pivot
+        for (int i = 0; i < n_; ++i)
+            if (eq_[i].mask >> var & 1) { eq_[i].mask ^= h.mask; eq_[i].value ^= h.value; again = true; }
+        if (again) reduce();
     }
 
     // One paired step: target bit t (s summed out, a' created), control bit c
-    // or -1. nz[c][a'][s]: the step's coefficient is not exactly zero.
-    void step(int t, int c, const bool (&nz)[2][2][2]) {
+    // or -1. Bit 4 c + 2 a' + s of nz: that coefficient is not exactly zero.
+    void step(int t, int c, unsigned nz) {
+        // bit i of ODD[m]: parity(i & m), i = 4 c + 2 a' + s
+        static constexpr unsigned ODD[8] = {0x00, 0xaa, 0xcc, 0x66, 0xf0, 0x5a, 0x3c, 0x96};
+        if (c < 0) nz &= 0x0f;
         const uint64_t tb = (uint64_t)1 << t, sb = (uint64_t)1 << TMP, cb = c < 0 ? 0 : (uint64_t)1 << c;
-        for (Eq& e : eq_)
-            if (e.mask & tb) { e.mask ^= tb | sb; e.pivot = TMP; }
-        std::vector<Eq> old;  // pivots moved with the rename: rebuild
-        old.swap(eq_);
-        for (const Eq& e : old) add(e.mask, e.value);
-        for (int m = 1; m < 8; ++m) {  // equations that every nonzero coefficient satisfies
-            if ((m & 4) && c < 0) continue;
-            int seen = 0;  // bit v: parity v occurs
-            for (int i = 0; i < 8; ++i) {
-                if (c < 0 && (i & 4)) continue;
-                if (nz[i >> 2][i >> 1 & 1][i & 1]) seen |= 1 << __builtin_parity(i & m);
-            }
-            if (seen == 1 || seen == 2)
-                add(((m & 4) ? cb : 0) | ((m & 2) ? tb : 0) | ((m & 1) ? sb : 0), seen == 2);
+        bool moved = false;
+        for (int i = 0; i < n_; ++i)
+            if (eq_[i].mask & tb) { eq_[i].mask ^= tb | sb; moved = true; }
+        if (moved) reduce();
+        bool more = false;
+        for (int m = 1; m < (c < 0 ? 4 : 8); ++m) {  // equations that every nonzero coefficient satisfies
+            const bool even = (nz & ~ODD[m]) != 0, odd = (nz & ODD[m]) != 0;
+            if (even == odd) continue;
+            add(((m & 4) ? cb : 0) | ((m & 2) ? tb : 0) | ((m & 1) ? sb : 0), odd);
+            more = true;
         }
-        eliminate(TMP);
+        if (moved || more) eliminate(TMP);
     }
 
-    // The tiles a pass visits: outside[i] is the address bit of tile-index bit
-    // i, in ascending order.
-    // At most max_n equations are used.
-    TileSkip skip(const std::vector<int>& outside, int h, int max_n = MAX_TILE_BITS) const {
-        Support s = *this;
-        uint64_t out = 0;
-        for (int b : outside) out |= (uint64_t)1 << b;
-        for (int b = 0; b < h; ++b)
-            if (!(out >> b & 1)) s.eliminate(b);
+    // The visited values of the address bits C.. without [lo, lo + M) (lo < 0:
+    // none left out): index bit i is the i-th of them. At most max_n equations
+    // are used; h: address bits in all.
+    TileSkip skip(int h, int C, int lo, int M, int max_n = MAX_TILE_BITS) const {
         TileSkip k;
         std::memset(&k, 0, sizeof(k));
-        const int nb = (int)outside.size();
-        auto index_mask = [&](uint64_t m) {
-            uint32_t r = 0;
-            for (int i = 0; i < nb; ++i)
-                if (m >> outside[i] & 1) r |= (uint32_t)1 << i;
-            return r;
-        };
-        if ((int)s.eq_.size() > max_n) s.eq_.resize(max_n);
+        if (lo < C) { lo = h; M = 0; }
+        const int nb = h - C - M;
+        if (nb > MAX_TILE_BITS) return k;  // wider than the device evaluates
+        Support s = *this;
+        for (int b = 0; b < C; ++b) s.eliminate(b);
+        for (int b = lo; b < lo + M; ++b) s.eliminate(b);
+        const uint64_t low = ((uint64_t)1 << (lo - C)) - 1;
+        auto index = [&](uint64_t m) { return (uint32_t)((m >> C & low) | (M ? m >> (lo + M) << (lo - C) : 0)); };
         // reduced equations: each pivot bit is determined by bits that are no pivots
-        uint32_t pivots = 0;
-        for (const Eq& e : s.eq_) {
-            const uint32_t pv = index_mask((uint64_t)1 << e.pivot);
-            pivots |= pv;
-            if (e.value) k.base |= pv;
-            ++k.n;
+        k.n = std::min(s.n_, max_n);
+        uint32_t mask[64], pivot[64], pivots = 0;
+        for (int e = 0; e < k.n; ++e) {
+            mask[e] = index(s.eq_[e].mask);
+            pivot[e] = index((uint64_t)1 << s.eq_[e].pivot);
+            pivots |= pivot[e];
+            if (s.eq_[e].value) k.base |= pivot[e];
         }
         for (int i = 0, u = 0; i < nb; ++i) {
             if (pivots >> i & 1) continue;
-            k.col[u] = (uint32_t)1 << i;
-            for (const Eq& e : s.eq_)
-                if (e.mask >> outside[i] & 1) k.col[u] |= index_mask((uint64_t)1 << e.pivot);
-            ++u;
+            uint32_t c = (uint32_t)1 << i;
+            for (int e = 0; e < k.n; ++e)
+                if (mask[e] >> i & 1) c |= pivot[e];
+            k.col[u++] = c;
         }
         return k;
     }
@@ -390,8 +383,12 @@ public:
     // The equation that determines bit var from the higher bits, if any (after the
     // lower bits have been eliminated): parity(address & *mask) ^ *value.
     bool determined(int var, uint64_t* mask, int* value) const {
-        for (const Eq& e : eq_)
-            if (e.mask >> var & 1) { *mask = e.mask & ~((uint64_t)1 << var); *value = e.value; return true; }
+        for (int i = 0; i < n_; ++i)
+            if (eq_[i].mask >> var & 1) {
+                *mask = eq_[i].mask & ~((uint64_t)1 << var);
+                *value = eq_[i].value;
+                return true;
+            }
         return false;
     }
 
@@ -400,61 +397,54 @@ private:
         uint64_t mask;
         int value, pivot;  // pivot: the highest variable, in no other equation
     };
-    std::vector<Eq> eq_;
+    void reduce() {  // bring the equations back into that form
+        Eq old[64];
+        const int n = n_;
+        std::copy(eq_, eq_ + n, old);
+        n_ = 0;
+        for (int i = 0; i < n; ++i) add(old[i].mask, old[i].value);
+    }
+    Eq eq_[64];  // independent, so at most one per variable
+    int n_ = 0;
 };
 
 // Fill in every pass's TileSkip. row0: the support of the row-0 boundary.
 static void tile_skips(Plan& P, Support s) {
     const int h = P.h;
-    bool finite = true;  // 0 x inf is not 0: such gates leave every tile visited
+    double z0 = 0.0;  // 0 x inf is not 0: non-finite gates leave every tile visited
     for (const auto& g : P.steps64)
-        for (const cd& z : g)
-            if (!std::isfinite(z.real()) || !std::isfinite(z.imag())) finite = false;
+        for (const cd& z : g) z0 += z.real() * 0.0 + z.imag() * 0.0;
+    const bool finite = z0 == 0.0;
+    if (!finite) s = Support();
     int done = 0;
     auto advance = [&](int end) {
-        for (; done < end; ++done) {
-            bool nz[2][2][2];
+        for (; finite && done < end; ++done) {
+            unsigned nz = 0;
             for (int i = 0; i < 8; ++i)  // of either output bit's variant
-                nz[i >> 2][i >> 1 & 1][i & 1] = P.steps64[done][i] != 0.0 || P.steps64[done][8 + i] != 0.0;
+                if (P.steps64[done][i] != 0.0 || P.steps64[done][8 + i] != 0.0) nz |= 1u << i;
             s.step(P.step_tgt[done], P.step_ctl[done], nz);
         }
     };
-    if (!finite) s = Support();
-    std::vector<int> outside;
     for (PassDesc& d : P.passes) {
-        const bool bottom = bottom_type(d.type);
-        const int C = bottom ? bot_chunk_bits(d.M) : high_low_bits(d.M);  // low address bits of a chunk
-        outside.clear();
-        for (int b = C; b < h; ++b)
-            if (bottom || b < d.lo || b >= d.lo + d.M) outside.push_back(b);
-        if ((int)outside.size() > MAX_TILE_BITS) continue;  // wider than the device evaluates
-        if (finite) advance(d.step0);
-        d.skip = s.skip(outside, h, h - TILE_BITS);  // at least one tile of visited chunks
+        advance(d.step0);
+        // outside the chunks; at least one tile of visited ones
+        d.skip = bottom_type(d.type) ? s.skip(h, bot_chunk_bits(d.M), -1, 0, h - TILE_BITS)
+                                     : s.skip(h, high_low_bits(d.M), d.lo, d.M, h - TILE_BITS);
     }
-    for (TcPass& d : P.tc_passes) {
-        outside.clear();
-        for (int b = 0, below = 0; b < h; ++b)
-            if (b < d.lo || b >= d.lo + P.tc_wb)
-                if (below++ >= TC_VEC_BITS) outside.push_back(b);
-        if ((int)outside.size() > MAX_TILE_BITS) continue;
-        if (finite) advance(d.step0);
-        d.skip = s.skip(outside, h);
+    for (TcPass& d : P.tc_passes) {  // outside the window and the TC_VEC_BITS lowest other bits
+        advance(d.step0);
+        d.skip = d.lo < TC_VEC_BITS ? s.skip(h, TC_VEC_BITS + P.tc_wb, -1, 0) : s.skip(h, TC_VEC_BITS, d.lo, P.tc_wb);
     }
-    auto above = [&](int lo) {
-        outside.clear();
-        for (int b = lo; b < h; ++b) outside.push_back(b);
-        return (int)outside.size() <= MAX_TILE_BITS;
-    };
-    if (finite) advance((int)P.steps.size());
+    advance((int)P.steps.size());
     if (!P.open_k) {
-        if (above(P.k)) P.red_skip = s.skip(outside, h);
+        P.red_skip = s.skip(h, P.k, -1, 0);
         return;
     }
     // open plan: the join mixes the k lowest bits, late crossing i sums bit k+i out
     const int k = P.open_k;
     P.late_skip.clear();
-    if (!above(k + 1)) s = Support();  // rows beyond the map: visit everything
-    if (above(k + 7)) P.join_skip = s.skip(outside, h);
+    if (h - k - 1 > MAX_TILE_BITS) s = Support();  // rows beyond the map: visit everything
+    P.join_skip = s.skip(h, k + 7, -1, 0);
     for (int b = 0; b < k; ++b) s.eliminate(b);
     for (size_t i = 0; i + 1 < P.open_seg.size(); ++i) {
         LateSkip ls;
@@ -467,8 +457,8 @@ static void tile_skips(Plan& P, Support s) {
         s.eliminate(k + (int)i);
         // the last crossing's output is read in full (2^k entries, or twice
         // that with an idle top bit)
-        if (above(k + (int)i + 1))
-            ls.out = i + 2 < P.open_seg.size() ? s.skip(outside, h) : Support().skip(outside, h);
+        ls.out = i + 2 < P.open_seg.size() ? s.skip(h, k + (int)i + 1, -1, 0)
+                                           : Support().skip(h, k + (int)i + 1, -1, 0);
         P.late_skip.push_back(ls);
     }
 }
