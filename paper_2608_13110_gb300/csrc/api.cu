@@ -215,6 +215,15 @@ int encode_join_map(CUtensorMap* m, const float2* base, int k, int64_t rows) {
     return TB_OK;
 }
 
+// Whether a pass gives each CTA a run of consecutive tiles instead of tiles
+// gridDim.x apart. A CTA that goes on to another bitstring flushes its maximum
+// and takes up a new scale, which runs make rare; tiles gridDim.x apart keep the
+// CTAs on neighbouring rows of HBM, which wide boundaries want. ms, apart ->
+// runs, dense gates: width 16, 200 bitstrings 1.70 -> 1.57; 20, 32: 5.17 ->
+// 4.95; 22, 32: 20.5 -> 20.1; 23, 32: 41.4 -> 41.0; 24, 32: 84.2 -> 84.4; 25,
+// 8: 44.2 -> 44.5.
+bool pass_runs(int tile_shift, int grid) { return ((int64_t)1 << tile_shift) < 8 * (int64_t)grid; }
+
 cudaError_t launch_pass(const PassDesc& d, const PassParams& p, const CUtensorMap& m, int grid, cudaStream_t st) {
     switch (d.type) {
         case P_FWD: return launch_pass_t0(d.M, p, m, grid, st);
@@ -356,6 +365,7 @@ int run_device(const Plan& P, const uint8_t* d_bits, int64_t nb, void* d_ws, int
             const int rc = encode_pass_map(&tmap, d, boundary, P.h, nbat);
             if (rc != TB_OK) return rc;
             const int grid = (int)std::min<int64_t>(pp.ntiles, (int64_t)PASS_CTAS_PER_SM * nsm);  // persistent CTAs
+            pp.runs = pass_runs(pp.tile_shift, grid) ? 1 : 0;
             ProfScope ps(PC_PASS, 16.0 * (double)nbat * (double)(b_stride >> d.skip.n), st);
             TB_CUDA(launch_pass(d, pp, tmap, grid, st));
         }
