@@ -163,7 +163,7 @@ EncodeTiledFn encode_tiled_fn() {
     return fn;
 }
 
-int encode_pass_map(CUtensorMap* m, const PassDesc& d, const float2* B, int h, int64_t nbatch) {
+int encode_pass_map(CUtensorMap* m, const PassDesc& d, const float2* B, int h, int64_t nbatch, bool small) {
     EncodeTiledFn enc = encode_tiled_fn();
     if (!enc) return fail(TB_ECUDA, "cuTensorMapEncodeTiled is not available from the driver");
     cuuint64_t dim[5];
@@ -171,15 +171,18 @@ int encode_pass_map(CUtensorMap* m, const PassDesc& d, const float2* B, int h, i
     cuuint32_t box[5];
     const cuuint32_t estr[5] = {1, 1, 1, 1, 1};
     const cuuint64_t E = 8;  // bytes per entry
+    int row = 128;           // bytes of a row of the stage
     if (bottom_type(d.type)) {
         const int CB = bot_chunk_bits(d.M);
         dim[0] = 32; dim[1] = (cuuint64_t)1 << (CB - 5); dim[2] = 2; dim[3] = (cuuint64_t)nbatch << (h - CB); dim[4] = 1;
         stride[0] = 32 * E; stride[1] = 16 * E; stride[2] = E << CB; stride[3] = E << CB;
         box[0] = 32; box[1] = (cuuint32_t)1 << (CB - 5); box[2] = 2; box[3] = 1; box[4] = 1;
     } else {
-        const int M = d.M, lo = d.lo, C = high_low_bits(M), W1 = M < 8 ? M : 8;
-        if (M < MIN_WINDOW || C < 3 || lo < C || lo + M > h) return fail(TB_EINVAL, "pass window outside the tensor-copy layout");
-        // 2^C entries per row (64 or 128 bytes), the window as 2^W1 x 2^(M-W1)
+        const int M = d.M, lo = d.lo, W1 = M < 8 ? M : 8;
+        const int C = high_low_bits(M) - (small ? small_row_log2(d.type, M) : 0);
+        if (M < MIN_WINDOW || C < 2 || lo < C || lo + M > h) return fail(TB_EINVAL, "pass window outside the tensor-copy layout");
+        // 2^C entries per row (32, 64 or 128 bytes), the window as 2^W1 x 2^(M-W1)
+        row = 8 << C;
         dim[0] = (cuuint64_t)2 << C; dim[1] = (cuuint64_t)1 << W1; dim[2] = (cuuint64_t)1 << (M - W1);
         dim[3] = (cuuint64_t)1 << (lo - C);
         dim[4] = (cuuint64_t)nbatch << (h - lo - M);
@@ -187,10 +190,12 @@ int encode_pass_map(CUtensorMap* m, const PassDesc& d, const float2* B, int h, i
         for (int i = 0; i < 3; ++i) box[i] = (cuuint32_t)dim[i];
         box[3] = 1; box[4] = 1;
     }
-    // rows of 64 bytes (a 10-bit window above bit 0) take the 64-byte swizzle
-    const bool row64 = !bottom_type(d.type) && TILE_BITS - d.M == 3;
+    // the swizzle spans a row
+    const CUtensorMapSwizzle swz = row == 128 ? CU_TENSOR_MAP_SWIZZLE_128B
+                                  : row == 64 ? CU_TENSOR_MAP_SWIZZLE_64B
+                                              : CU_TENSOR_MAP_SWIZZLE_32B;
     const CUresult r = enc(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 5, const_cast<float2*>(B), dim, stride, box, estr,
-                           CU_TENSOR_MAP_INTERLEAVE_NONE, row64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B,
+                           CU_TENSOR_MAP_INTERLEAVE_NONE, swz,
                            CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS)
         return fail(TB_ECUDA, "cuTensorMapEncodeTiled failed (" + std::to_string((int)r) + ") for a pass of type " +
@@ -213,6 +218,14 @@ int encode_join_map(CUtensorMap* m, const float2* base, int k, int64_t rows) {
     if (r != CUDA_SUCCESS)
         return fail(TB_ECUDA, "cuTensorMapEncodeTiled failed for the join (" + std::to_string((int)r) + ")");
     return TB_OK;
+}
+
+// Whether a pass runs on small tiles, one per CTA: as long as they fit on the
+// device at once. With the 8 to 32 tiles of a single narrow bitstring, whole
+// tiles leave most SMs idle while 8 warps share one (n=33, d=35, one bitstring:
+// 410 -> 364 us).
+bool small_tiles(const PassDesc& d, int64_t ntiles, int nsm) {
+    return has_small_tiles(d.type, d.M) && (ntiles << SMALL_TILE_LOG2) <= (int64_t)SMALL_CTAS_PER_SM * nsm;
 }
 
 // Whether a pass gives each CTA a run of consecutive tiles instead of tiles
@@ -361,10 +374,15 @@ int run_device(const Plan& P, const uint8_t* d_bits, int64_t nb, void* d_ws, int
             pp.slot = (int)k;
             pp.fault = fault;
             pp.selftest = t_pass_selftest ? 1 : 0;
+            pp.small = small_tiles(d, pp.ntiles, nsm) ? 1 : 0;
+            if (pp.small) {
+                pp.tile_shift += SMALL_TILE_LOG2;
+                pp.ntiles <<= SMALL_TILE_LOG2;
+            }
             CUtensorMap tmap;
-            const int rc = encode_pass_map(&tmap, d, boundary, P.h, nbat);
+            const int rc = encode_pass_map(&tmap, d, boundary, P.h, nbat, pp.small != 0);
             if (rc != TB_OK) return rc;
-            const int grid = (int)std::min<int64_t>(pp.ntiles, (int64_t)PASS_CTAS_PER_SM * nsm);  // persistent CTAs
+            const int grid = pp.small ? (int)pp.ntiles : (int)std::min<int64_t>(pp.ntiles, (int64_t)PASS_CTAS_PER_SM * nsm);
             pp.runs = pass_runs(pp.tile_shift, grid) ? 1 : 0;
             ProfScope ps(PC_PASS, 16.0 * (double)nbat * (double)(b_stride >> d.skip.n), st);
             TB_CUDA(launch_pass(d, pp, tmap, grid, st));

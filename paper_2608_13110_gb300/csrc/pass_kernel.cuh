@@ -55,6 +55,7 @@ struct PassParams {
     int tile_shift;       // log2(tiles visited per batch element) = h - TILE_BITS - skip.n
     int64_t ntiles;       // nbatch << tile_shift
     int runs;             // 1: a CTA works on consecutive tiles, 0: on tiles gridDim.x apart
+    int small;            // 1: small tiles (ntiles and tile_shift count them; the host's choice of kernel)
     TileSkip skip;        // which tiles are visited
     const StepG* steps;   // the pass's first step
     int xs_step0, xs_q0, xs_step1, xs_q1;
@@ -85,30 +86,39 @@ __device__ __forceinline__ uint32_t pass_smem_u32(const void* p) {
 //     8..12, the warp index 0..2.
 // Every window bit is a lane or register bit in each case.
 constexpr int LAY_BOT = 0, LAY_HIGH = 1, LAY_LOW3 = 2;
-template <int TYPE_, int M_>
+template <int TYPE_, int M_, bool SMALL_>
 struct Shape {
     static constexpr int TYPE = TYPE_;
     static constexpr int M = M_;
+    static constexpr bool SMALL = SMALL_;                 // quarter tiles: 2 consumer warps
+    static constexpr int WARPS = SMALL ? 2 : 8;
+    static constexpr int CONSUMERS = 32 * WARPS;
+    static constexpr int THREADS = SMALL ? CONSUMERS + 32 : PASS_THREADS;
+    static constexpr int STAGES = SMALL ? 1 : 3;          // small tiles: one per CTA
+    static constexpr int ENTRIES = 1024 * WARPS;
+    static constexpr int ROWL = SMALL ? small_row_log2(TYPE, M) : 0;  // log2 of the parts of a row
     static constexpr bool BOT = bottom_type(TYPE);
     static constexpr int NS = pass_nsteps(TYPE, M);
     static constexpr int XM = pass_xm(TYPE, M);           // step with four variants (-1: none)
     static constexpr int BLK = pass_blk(TYPE, M);         // the turn's 4x4 block (-1: none)
     static constexpr int NB = 2 * NS + (XM >= 0 ? 2 : 0);  // coefficient blocks
-    static constexpr int C = BOT ? 0 : high_low_bits(M);  // tile bit of window bit 0
+    static constexpr int C = BOT ? 0 : high_low_bits(M) - ROWL;  // tile bit of window bit 0
     static constexpr int CB = BOT ? bot_chunk_bits(M) : 0;
-    static constexpr int CHL = pass_chunk_log2(TYPE, M);  // log2 of the chunks of a tile
-    static constexpr int LAY = BOT ? LAY_BOT : (C == 3 ? LAY_LOW3 : LAY_HIGH);
+    static constexpr int CHL = pass_chunk_log2(TYPE, M) - (SMALL ? SMALL_TILE_LOG2 - ROWL : 0);  // log2 of the chunks of a tile
+    static constexpr int LAY = BOT ? LAY_BOT : (M > 9 ? LAY_LOW3 : LAY_HIGH);
+    static constexpr int SWZ = BOT || C == 4 ? 128 : (C == 3 ? 64 : 32);  // bytes of a row of the stage
     static constexpr int REG0 = BOT ? 5 : C + M - REG_BITS;  // tile bit of register bit 0
     static constexpr int regpos(int t) { return (t >= REG0 && t < REG0 + REG_BITS) ? t - REG0 : -1; }
     static constexpr int lanepos(int t) {
         if (BOT) return t < 5 ? t : -1;
         if (LAY == LAY_LOW3) return (t >= 3 && t < 8) ? t - 3 : -1;
-        return t == 0 ? 0 : (t >= 4 && t < REG0) ? t - 3 : -1;
+        return t == 0 ? 0 : (t >= C && t < REG0) ? t - C + 1 : -1;
     }
     static constexpr int tgt(int i) { return C + step_spec(TYPE, M, i).t; }
     static constexpr int ctl(int i) { return step_spec(TYPE, M, i).c < 0 ? -1 : C + step_spec(TYPE, M, i).c; }
     static constexpr bool valid() {
         if (M < MIN_WINDOW || M > (BOT ? MAX_WINDOW : MAX_WINDOW_HIGH)) return false;
+        if (SMALL && !has_small_tiles(TYPE, M)) return false;
         for (int j = 0; j < NS; ++j) {
             if (j == BLK) {  // bottom: lanes 0, 1 with control lane 2; top: registers 3, 4 with control register 2
                 if (BOT ? (lanepos(tgt(j)) != 0 || lanepos(tgt(j) + 1) != 1 || lanepos(ctl(j)) != 2)
@@ -136,9 +146,15 @@ __device__ __forceinline__ uint32_t thread_base(uint32_t tid) {
                                 {0, 4, 5, 3, 1, 2, 11, 12},    // 7
                                 {0, 4, 5, 6, 1, 2, 3, 12},     // 8
                                 {0, 4, 5, 6, 7, 1, 2, 3}};     // 9
+    constexpr int SBITS[5][6] = {{0, 1, 2, 3, 9, 10},  // small tiles; M = 8 and 9 hold 3 and 2 low address bits
+                                 {0, 4, 2, 3, 1, 10},
+                                 {0, 4, 5, 3, 1, 2},
+                                 {0, 3, 4, 5, 1, 2},
+                                 {0, 2, 3, 4, 5, 1}};
     uint32_t b = 0;
 #pragma unroll
-    for (int i = 0; i < 8; ++i) b |= (tid >> i & 1u) << BITS[SH::M < 9 ? SH::M - 5 : 4][i];
+    for (int i = 0; i < (SH::SMALL ? 6 : 8); ++i)
+        b |= (tid >> i & 1u) << (SH::SMALL ? SBITS[SH::M < 9 ? SH::M - 5 : 4][i < 6 ? i : 0] : BITS[SH::M < 9 ? SH::M - 5 : 4][i]);
     return b;
 }
 
@@ -157,6 +173,9 @@ __device__ __forceinline__ uint32_t thread_base(uint32_t tid) {
 //     5..CB-1, then 4; then the chunk (tile bits CB..12). Lanes 0..3 hold
 //     tile bits 0..3 and registers bits 5..7, so the swizzled bits are
 //     t0, t1^t5, t2^t6, t3^t7: again a bijection of the lane bits.
+//   * small tiles of 8- and 9-bit windows: identity order in rows of 64 and 32
+//     bytes with their swizzles; lanes 0..3 again reach four different bank
+//     bits (M = 8: t0, t3, t4 -> 1, t5 -> 2; M = 9: t0, t2, t3, t4 -> 1).
 //   * 10-bit windows above bit 0 (LAY_LOW3): identity order in rows of 64
 //     bytes with the 64-byte swizzle (slot bits 1..2 ^= 4..5). Slot bit 0 is
 //     the warp's tile bit 0, so a half warp's 16 slots cover 8 bank pairs:
@@ -167,21 +186,23 @@ __device__ __forceinline__ uint32_t thread_base(uint32_t tid) {
 // ---------------------------------------------------------------------------
 __host__ __device__ constexpr uint32_t swz128(uint32_t s) { return s ^ (((s >> 4) & 7u) << 1); }
 
-// 64-byte swizzle (rows of 64 bytes, LAY_LOW3): slot bits 1..2 ^= 4..5.
+// Rows of 64 bytes: slot bits 1..2 ^= 4..5; of 32 bytes: slot bit 1 ^= 4.
 __host__ __device__ constexpr uint32_t swz64(uint32_t s) { return s ^ (((s >> 4) & 3u) << 1); }
+__host__ __device__ constexpr uint32_t swz32(uint32_t s) { return s ^ (((s >> 4) & 1u) << 1); }
 
-template <int LAY, int CB>
+template <class SH>
 __host__ __device__ constexpr uint32_t slot_of(uint32_t idx) {
-    if (LAY == LAY_LOW3) return swz64(idx);
-    constexpr uint32_t MID = LAY == LAY_BOT ? (1u << (CB - 5)) - 1u : 0u;  // bits 5..CB-1
-    return swz128(LAY == LAY_BOT ? ((idx & 15u) | (((idx >> 5) & MID) << 4) | (((idx >> 4) & 1u) << (CB - 1)) |
-                                    ((idx >> CB) << CB))
-                                 : idx);
+    if (SH::SWZ == 64) return swz64(idx);
+    if (SH::SWZ == 32) return swz32(idx);
+    constexpr uint32_t MID = SH::BOT ? (1u << (SH::CB - 5)) - 1u : 0u;  // bits 5..CB-1
+    return swz128(SH::BOT ? ((idx & 15u) | (((idx >> 5) & MID) << 4) | (((idx >> 4) & 1u) << (SH::CB - 1)) |
+                             ((idx >> SH::CB) << SH::CB))
+                          : idx);
 }
 
-template <int LAY, int CB, uint32_t J>
+template <class SH, uint32_t J>
 struct SlotC {
-    static constexpr uint32_t v = slot_of<LAY, CB>(J);
+    static constexpr uint32_t v = slot_of<SH>(J);
 };
 
 // ---------------------------------------------------------------------------
@@ -375,7 +396,7 @@ __host__ __device__ constexpr uint64_t step_kinds() {
 template <class SH>
 __device__ __forceinline__ void stage_coefficients(const StepG* steps, float2* sc, uint32_t tid) {
     constexpr uint64_t KINDS = step_kinds<SH>();
-    for (int w = tid; w < SH::NB; w += PASS_THREADS) {
+    for (int w = tid; w < SH::NB; w += SH::THREADS) {
         const int i = w < 2 * SH::NS ? w >> 1 : SH::XM, x = w & 1;
         float2* o = sc + w * CO;
         for (int e = 0; e < CO; ++e) o[e] = make_float2(0.f, 0.f);
@@ -452,23 +473,23 @@ __device__ __forceinline__ void stage_coefficients(const StepG* steps, float2* s
 
 // Registers <-> shared stage: entry j of a thread sits at tile coordinate
 // thread_base | j << REG0, i.e. slot base ^ SlotC<j << REG0>.
-template <int LAY, int CB, int REG0, int J>
+template <class SH, int J>
 __device__ __forceinline__ void smem_read_j(float2 (&P)[16], float2 (&Q)[16], const float2* tile, uint32_t sb) {
     if constexpr (J < 32) {
-        const float2 e = tile[sb ^ SlotC<LAY, CB, ((uint32_t)J << REG0)>::v];
+        const float2 e = tile[sb ^ SlotC<SH, ((uint32_t)J << SH::REG0)>::v];
         if constexpr (J < 16) { P[J].x = e.x; Q[J].x = e.y; }
         else                  { P[J - 16].y = e.x; Q[J - 16].y = e.y; }
-        smem_read_j<LAY, CB, REG0, J + 1>(P, Q, tile, sb);
+        smem_read_j<SH, J + 1>(P, Q, tile, sb);
     }
 }
 
-template <int LAY, int CB, int REG0, int J>
+template <class SH, int J>
 __device__ __forceinline__ void smem_write_j(const float2 (&P)[16], const float2 (&Q)[16], float2* tile,
                                              uint32_t sb) {
     if constexpr (J < 32) {
-        tile[sb ^ SlotC<LAY, CB, ((uint32_t)J << REG0)>::v] =
+        tile[sb ^ SlotC<SH, ((uint32_t)J << SH::REG0)>::v] =
             J < 16 ? make_float2(P[J & 15].x, Q[J & 15].x) : make_float2(P[J & 15].y, Q[J & 15].y);
-        smem_write_j<LAY, CB, REG0, J + 1>(P, Q, tile, sb);
+        smem_write_j<SH, J + 1>(P, Q, tile, sb);
     }
 }
 
@@ -617,7 +638,8 @@ __device__ __forceinline__ void tile_coords(const PassParams& p, int64_t gt, uin
                                             uint32_t chunk, int& c3, int& c4) {
     const int64_t b = gt >> p.tile_shift;
     const uint32_t u = (uint32_t)(gt & (((int64_t)1 << p.tile_shift) - 1));
-    const int64_t t = tile_of_warp(p.skip.base, col, lane, u << SH::CHL) ^ chunk;
+    int64_t t = tile_of_warp(p.skip.base, col, lane, (u >> SH::ROWL) << SH::CHL) ^ chunk;
+    if constexpr (SH::ROWL > 0) t = (t << SH::ROWL) | (u & ((1u << SH::ROWL) - 1u));  // part of the rows
     if constexpr (SH::BOT) {
         c3 = (int)((b << (p.h - SH::CB)) + t);
         c4 = 0;
@@ -628,29 +650,26 @@ __device__ __forceinline__ void tile_coords(const PassParams& p, int64_t gt, uin
     }
 }
 
-constexpr int PASS_STAGES = 3;
-constexpr uint32_t TILE_BYTES = (uint32_t)TILE * 8u;
-
-template <int TYPE, int M>
+template <class SH>
 constexpr int pass_smem_bytes() {
-    return 1024 + PASS_STAGES * TILE * 8 + Shape<TYPE, M>::NB * CO * 8 + 2 * PASS_STAGES * 8 + 16;
+    return 1024 + SH::STAGES * SH::ENTRIES * 8 + SH::NB * CO * 8 + 2 * SH::STAGES * 8 + 16;
 }
 
-template <int TYPE, int M>
-__global__ void __launch_bounds__(PASS_THREADS, PASS_CTAS_PER_SM)
+template <class SH>
+__global__ void __launch_bounds__(SH::THREADS, SH::SMALL ? SMALL_CTAS_PER_SM : PASS_CTAS_PER_SM)
     pass_kernel(const __grid_constant__ PassParams p, const __grid_constant__ CUtensorMap tmap) {
-    using SH = Shape<TYPE, M>;
     static_assert(SH::valid(), "invalid pass shape");
     static_assert(SH::NS <= XM_HIGH_BIT, "variant mask: one bit per step, bit XM_HIGH_BIT for the four-variant step");
-    constexpr int NS = SH::NS;
+    constexpr int STAGES = SH::STAGES;
+    constexpr uint32_t TILE_BYTES = SH::ENTRIES * 8u;
     extern __shared__ __align__(16) uint8_t dsm[];
     uint8_t* base = dsm + ((1024u - (pass_smem_u32(dsm) & 1023u)) & 1023u);
     float2* stages = reinterpret_cast<float2*>(base);
-    float2* sc = stages + PASS_STAGES * TILE;
+    float2* sc = stages + STAGES * SH::ENTRIES;
     uint64_t* bars = reinterpret_cast<uint64_t*>(sc + SH::NB * CO);  // full[3], done[3]
-    int* s_abort = reinterpret_cast<int*>(bars + 2 * PASS_STAGES);
+    int* s_abort = reinterpret_cast<int*>(bars + 2 * STAGES);
     const uint32_t tid = threadIdx.x;
-    const uint32_t full0 = pass_smem_u32(bars), done0 = full0 + 8 * PASS_STAGES;
+    const uint32_t full0 = pass_smem_u32(bars), done0 = full0 + 8 * STAGES;
     const uint32_t stage0 = pass_smem_u32(stages);
 
     // tiles first, first + step, ... of this CTA (grid <= ntiles)
@@ -670,17 +689,17 @@ __global__ void __launch_bounds__(PASS_THREADS, PASS_CTAS_PER_SM)
         const uint32_t ci = __shfl_sync(0xffffffffu, col, i);
         if (lane >> i & 1u) chunk ^= ci;
     }
-    int t3[PASS_STAGES], t4[PASS_STAGES];  // producer: coordinates of the tile in each stage
+    int t3[STAGES], t4[STAGES];  // producer: coordinates of the tile in each stage
 
     // The producer warp (the first of the last warpgroup) works on tile
     // coordinates together; its lane 0 sets the barriers up and issues every
     // copy. The first loads do not wait for the coefficients.
-    if ((tid >> 5) == PASS_CONSUMERS / 32) {
+    if ((tid >> 5) == SH::WARPS) {
         if (lane == 0) {
             asm volatile("prefetch.tensormap [%0];\n" ::"l"(reinterpret_cast<uint64_t>(&tmap)) : "memory");
-            for (int s = 0; s < PASS_STAGES; ++s) {
+            for (int s = 0; s < STAGES; ++s) {
                 pbar_init(full0 + 8 * s, 1);
-                pbar_init(done0 + 8 * s, PASS_CONSUMERS / 32);
+                pbar_init(done0 + 8 * s, SH::WARPS);
             }
             *s_abort = 0;
             asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
@@ -688,7 +707,7 @@ __global__ void __launch_bounds__(PASS_THREADS, PASS_CTAS_PER_SM)
         }
         grid_wait();
         if (!p.selftest)
-            for (int k = 0; k < ntl && k < PASS_STAGES; ++k) {
+            for (int k = 0; k < ntl && k < STAGES; ++k) {
                 tile_coords<SH>(p, first + k * step, col, lane, chunk, t3[k], t4[k]);
                 if (lane == 0) pbar_expect_tx(full0 + 8 * k, TILE_BYTES);
                 __syncwarp();
@@ -712,55 +731,55 @@ __global__ void __launch_bounds__(PASS_THREADS, PASS_CTAS_PER_SM)
     static_assert((PASS_THREADS - PASS_CONSUMERS) * PASS_PRODUCER_REGS + PASS_CONSUMERS * PASS_CONSUMER_REGS <=
                       PASS_THREADS * (65536 / PASS_THREADS / 8 * 8),
                   "register split exceeds the launch's registers");
-    if (tid >= PASS_CONSUMERS) {
-        // ---------------- producer: one warp of the last warpgroup
-        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;\n" ::"n"(PASS_PRODUCER_REGS));
-        if ((tid >> 5) != PASS_CONSUMERS / 32) return;
-        int64_t last_load[PASS_STAGES];  // tile index k of the latest load per stage (-1: none)
-        for (int st = 0; st < PASS_STAGES; ++st) last_load[st] = !p.selftest && st < ntl ? st : -1;
+    if (tid >= SH::CONSUMERS) {
+        // ---------------- producer: one warp (of the last warpgroup)
+        if constexpr (!SH::SMALL) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;\n" ::"n"(PASS_PRODUCER_REGS));
+        if ((tid >> 5) != SH::WARPS) return;
+        int64_t last_load[STAGES];  // tile index k of the latest load per stage (-1: none)
+        for (int st = 0; st < STAGES; ++st) last_load[st] = !p.selftest && st < ntl ? st : -1;
         int s = 0;
         uint32_t ph = 0;
         for (int64_t k = 0; k < ntl; ++k) {
             int n3 = 0, n4 = 0;  // the stage's next tile, worked out while the consumers are busy
-            if (k + PASS_STAGES < ntl) tile_coords<SH>(p, first + (k + PASS_STAGES) * step, col, lane, chunk, n3, n4);
+            if (k + STAGES < ntl) tile_coords<SH>(p, first + (k + STAGES) * step, col, lane, chunk, n3, n4);
             const bool gave_up = !pbar_wait(done0 + 8 * s, ph, tries);
             if (__any_sync(0xffffffffu, gave_up)) {
                 if (lane == 0 && atomicExch(s_abort, 1) == 0) atomicAdd(p.fault, 1);
                 break;
             }
             if (mover) tma_store_tile(&tmap, t3[s], t4[s], stage0 + (uint32_t)s * TILE_BYTES + lane * PART);
-            if (k + PASS_STAGES < ntl) {
+            if (k + STAGES < ntl) {
                 if (mover) tma_wait_read_all();  // the stores have read the stage
                 if (lane == 0) pbar_expect_tx(full0 + 8 * s, TILE_BYTES);
                 __syncwarp();
                 if (mover) tma_load_tile(stage0 + (uint32_t)s * TILE_BYTES + lane * PART, &tmap, n3, n4, full0 + 8 * s);
-                last_load[s] = k + PASS_STAGES;
+                last_load[s] = k + STAGES;
                 t3[s] = n3;
                 t4[s] = n4;
             }
             __syncwarp();
-            if (++s == PASS_STAGES) { s = 0; ph ^= 1u; }
+            if (++s == STAGES) { s = 0; ph ^= 1u; }
         }
         if (mover) tma_wait_all();
         __syncwarp();
         if (lane == 0 && *(volatile int*)s_abort) {
             // loads still in flight must land before the CTA's shared memory goes
-            for (int st = 0; st < PASS_STAGES; ++st)
+            for (int st = 0; st < STAGES; ++st)
                 if (last_load[st] >= 0)
-                    (void)pbar_wait(full0 + 8 * st, (uint32_t)((last_load[st] / PASS_STAGES) & 1), PASS_WAIT_TRIES);
+                    (void)pbar_wait(full0 + 8 * st, (uint32_t)((last_load[st] / STAGES) & 1), PASS_WAIT_TRIES);
         }
         return;
     }
 
-    // ---------------- consumers (tid < 256): 8 independent warps
-    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;\n" ::"n"(PASS_CONSUMER_REGS));
+    // ---------------- consumers: 8 (small tiles: 2) independent warps
+    if constexpr (!SH::SMALL) asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;\n" ::"n"(PASS_CONSUMER_REGS));
     float runmax = 0.0f;
     int64_t cur_b = -1;
     int cur_s = 0;
     float scale = 1.0f;
     uint32_t xmask = 0;
     const int64_t tmask = ((int64_t)1 << p.tile_shift) - 1;
-    const uint32_t sb = slot_of<SH::LAY, SH::CB>(thread_base<SH>(tid));
+    const uint32_t sb = slot_of<SH>(thread_base<SH>(tid));
     // A bitstring's rescaling maximum and output bits, read while the tile before
     // its first one is worked on: reading the state on the spot put two global
     // latencies into every change of bitstring (n=61, d=32, 200 bitstrings: 3.90
@@ -802,18 +821,18 @@ __global__ void __launch_bounds__(PASS_THREADS, PASS_CTAS_PER_SM)
         }
         if (t == 0 && tid == 0) p.exps[b * p.sstride + p.slot + 1] = cur_s;
 
-        float2* tile = stages + s * TILE;
+        float2* tile = stages + s * SH::ENTRIES;
         float2 P[16], Q[16];
-        smem_read_j<SH::LAY, SH::CB, SH::REG0, 0>(P, Q, tile, sb);
+        smem_read_j<SH, 0>(P, Q, tile, sb);
         run_steps<SH, 0>(P, Q, sc, xmask, scale, tid);
 #pragma unroll
         for (int j = 0; j < 16; ++j)
             runmax = fmaxf(runmax, fmaxf(fmaxf(fabsf(P[j].x), fabsf(P[j].y)), fmaxf(fabsf(Q[j].x), fabsf(Q[j].y))));
-        smem_write_j<SH::LAY, SH::CB, SH::REG0, 0>(P, Q, tile, sb);
+        smem_write_j<SH, 0>(P, Q, tile, sb);
         asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");  // visible to the tensor store
         __syncwarp();
         if ((tid & 31u) == 0) pbar_arrive(done0 + 8 * s);
-        if (++s == PASS_STAGES) { s = 0; ph ^= 1u; }
+        if (++s == STAGES) { s = 0; ph ^= 1u; }
     }
     if (cur_b >= 0) flush_max(runmax, p.maxs + cur_b * p.sstride + p.slot + 1);
     if (!one_tile) grid_release();
@@ -828,17 +847,22 @@ cudaError_t launch_pass_t4(int M, const PassParams& p, const CUtensorMap& m, int
 cudaError_t launch_pass_t5(int M, const PassParams& p, const CUtensorMap& m, int grid, cudaStream_t st);
 cudaError_t launch_pass_t6(int M, const PassParams& p, const CUtensorMap& m, int grid, cudaStream_t st);
 
-template <int TYPE, int M>
-cudaError_t launch_one(const PassParams& p, const CUtensorMap& m, int grid, cudaStream_t st) {
-    if constexpr (!Shape<TYPE, M>::valid()) {
+template <class SH>
+cudaError_t launch_shape(const PassParams& p, const CUtensorMap& m, int grid, cudaStream_t st) {
+    if constexpr (!SH::valid()) {
         return cudaErrorInvalidValue;
     } else {
-        constexpr int smem = pass_smem_bytes<TYPE, M>();
+        constexpr int smem = pass_smem_bytes<SH>();
         static_assert(smem <= 227 * 1024, "pass kernel shared memory");
-        cudaError_t e = cudaFuncSetAttribute(pass_kernel<TYPE, M>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        cudaError_t e = cudaFuncSetAttribute(pass_kernel<SH>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         if (e != cudaSuccess) return e;
-        return launch_after(pass_kernel<TYPE, M>, grid, PASS_THREADS, smem, st, p, m);
+        return launch_after(pass_kernel<SH>, grid, SH::THREADS, smem, st, p, m);
     }
+}
+
+template <int TYPE, int M>
+cudaError_t launch_one(const PassParams& p, const CUtensorMap& m, int grid, cudaStream_t st) {
+    return p.small ? launch_shape<Shape<TYPE, M, true>>(p, m, grid, st) : launch_shape<Shape<TYPE, M, false>>(p, m, grid, st);
 }
 
 #define TB_DEFINE_LAUNCH_PASS(TYPE, NAME)                                                      \

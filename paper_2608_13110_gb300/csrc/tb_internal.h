@@ -16,6 +16,7 @@ constexpr int PASS_THREADS = PASS_CONSUMERS + 128;  // + one producer warpgroup 
 constexpr int PASS_PRODUCER_REGS = 40;   // setmaxnreg split of the 168 registers per thread at launch:
 constexpr int PASS_CONSUMER_REGS = 224;  // 128 x 40 + 256 x 224 <= 384 x 168
 constexpr int PASS_CTAS_PER_SM = 1;
+constexpr int SMALL_CTAS_PER_SM = 3;  // of small tiles (96 threads of at most 224 registers)
 constexpr int REG_BITS = 5;           // entries per thread = 2^REG_BITS
 constexpr int MIN_WINDOW = 5;
 constexpr int MAX_WINDOW = 10;        // window at address bit 0 (whole tile is low bits)
@@ -174,6 +175,17 @@ __host__ __device__ constexpr bool bottom_type(int type) {
 __host__ __device__ constexpr int pass_chunk_log2(int type, int M) {
     return TILE_BITS - (bottom_type(type) ? bot_chunk_bits(M) : M + high_low_bits(M));
 }
+
+// Small tiles, for launches that would leave SMs idle: a quarter of a tile, the
+// entries of 2 of its 8 consumer warps (each warp's steps are the same). Quarter
+// q of a tile: the chunks with q as their number's two highest bits, or, where a
+// tile has fewer than four chunks, part of every row (log2 of the parts:
+// small_row_log2). 10-bit windows above bit 0 have none.
+constexpr int SMALL_TILE_LOG2 = 2;
+__host__ __device__ constexpr int small_row_log2(int type, int M) {
+    return pass_chunk_log2(type, M) < SMALL_TILE_LOG2 ? SMALL_TILE_LOG2 - pass_chunk_log2(type, M) : 0;
+}
+__host__ __device__ constexpr bool has_small_tiles(int type, int M) { return bottom_type(type) || M <= 9; }
 
 // Rows of a late crossing of an open plan: output rows visited, and which of
 // the input rows 2r', 2r'+1 may be nonzero (one: both == 0, the row whose low
