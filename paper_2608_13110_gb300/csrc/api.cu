@@ -190,13 +190,14 @@ int encode_pass_map(CUtensorMap* m, const PassDesc& d, const float2* B, int h, i
         for (int i = 0; i < 3; ++i) box[i] = (cuuint32_t)dim[i];
         box[3] = 1; box[4] = 1;
     }
-    // the swizzle spans a row
+    // The swizzle spans a row. Promotion to 256 bytes would fetch neighbouring rows
+    // that a pass may leave out (n=70, d=56, two bitstrings: 134.2 ms, 131.9 with 128).
     const CUtensorMapSwizzle swz = row == 128 ? CU_TENSOR_MAP_SWIZZLE_128B
                                   : row == 64 ? CU_TENSOR_MAP_SWIZZLE_64B
                                               : CU_TENSOR_MAP_SWIZZLE_32B;
     const CUresult r = enc(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 5, const_cast<float2*>(B), dim, stride, box, estr,
                            CU_TENSOR_MAP_INTERLEAVE_NONE, swz,
-                           CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+                           CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS)
         return fail(TB_ECUDA, "cuTensorMapEncodeTiled failed (" + std::to_string((int)r) + ") for a pass of type " +
                                   std::to_string(d.type) + ", M=" + std::to_string(d.M) + ", lo=" + std::to_string(d.lo));
