@@ -365,6 +365,7 @@ int run_device(const Plan& P, const uint8_t* d_bits, int64_t nb, void* d_ws, int
             pp.tile_shift = P.h - TILE_BITS - d.skip.n;
             pp.ntiles = (int64_t)nbat << pp.tile_shift;
             pp.skip = d.skip;
+            pp.warps = d.warps;
             pp.steps = pass_steps + d.pstep0;
             pp.xs_step0 = d.xs_step[0]; pp.xs_q0 = d.xs_q[0];
             pp.xs_step1 = d.xs_step[1]; pp.xs_q1 = d.xs_q[1];

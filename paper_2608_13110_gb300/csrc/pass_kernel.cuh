@@ -57,6 +57,7 @@ struct PassParams {
     int runs;             // 1: a CTA works on consecutive tiles, 0: on tiles gridDim.x apart
     int small;            // 1: small tiles (ntiles and tile_shift count them; the host's choice of kernel)
     TileSkip skip;        // which tiles are visited
+    WarpSkip warps;       // and which of their warps have something to do
     const StepG* steps;   // the pass's first step
     int xs_step0, xs_q0, xs_step1, xs_q1;
     const uint8_t* bits;  // bitstring of batch element b at bits + b*n
@@ -86,11 +87,12 @@ __device__ __forceinline__ uint32_t pass_smem_u32(const void* p) {
 //     8..12, the warp index 0..2.
 // Every window bit is a lane or register bit in each case.
 constexpr int LAY_BOT = 0, LAY_HIGH = 1, LAY_LOW3 = 2;
-template <int TYPE_, int M_, bool SMALL_>
+template <int TYPE_, int M_, bool SMALL_, bool ZW_ = false>
 struct Shape {
     static constexpr int TYPE = TYPE_;
     static constexpr int M = M_;
     static constexpr bool SMALL = SMALL_;                 // quarter tiles: 2 consumer warps
+    static constexpr bool ZW = ZW_;                       // leaves zero warps out (WarpSkip)
     static constexpr int WARPS = SMALL ? 2 : 8;
     static constexpr int CONSUMERS = 32 * WARPS;
     static constexpr int THREADS = SMALL ? CONSUMERS + 32 : PASS_THREADS;
@@ -650,6 +652,15 @@ __device__ __forceinline__ void tile_coords(const PassParams& p, int64_t gt, uin
     }
 }
 
+// Tile-map columns of the chunk that warp w works on (8-bit windows: two chunks
+// per tile, the warp index's highest bit; 9-bit windows: one).
+template <class SH>
+__device__ __forceinline__ uint32_t chunk_of_warp(uint32_t col, uint32_t w) {
+    if constexpr (SH::CHL == 0) return 0u;
+    const uint32_t c0 = __shfl_sync(0xffffffffu, col, 0);
+    return w >> 2 & 1u ? c0 : 0u;
+}
+
 template <class SH>
 constexpr int pass_smem_bytes() {
     return 1024 + SH::STAGES * SH::ENTRIES * 8 + SH::NB * CO * 8 + 2 * SH::STAGES * 8 + 16;
@@ -779,7 +790,24 @@ __global__ void __launch_bounds__(SH::THREADS, SH::SMALL ? SMALL_CTAS_PER_SM : P
     float scale = 1.0f;
     uint32_t xmask = 0;
     const int64_t tmask = ((int64_t)1 << p.tile_shift) - 1;
-    const uint32_t sb = slot_of<SH>(thread_base<SH>(tid));
+    uint32_t sb = slot_of<SH>(thread_base<SH>(tid));
+    // Zero warps: a warp whose 1024 entries are zero passes the tile on. Which
+    // they are changes with the tile at most through its address, so the warps
+    // take turns (warp w works as warp w ^ k on tile k): otherwise the same
+    // schedulers would idle in every tile. n=61, d=32, 200 bitstrings 3.54 ->
+    // 3.33 ms. A kernel of its own: in the common one it took 2 % of the passes
+    // without zero warps.
+    uint32_t wout = 0, wmask = 0;
+    uint32_t wslot[3] = {0, 0, 0};
+    if constexpr (SH::ZW) {
+        if (lane < (uint32_t)p.warps.n) {
+            wout = p.warps.out[lane];
+            wmask = p.warps.warp[lane];
+        }
+#pragma unroll
+        for (int i = 0; i < 3; ++i) wslot[i] = slot_of<SH>(thread_base<SH>(32u << i));
+    }
+    const uint32_t sb0 = sb;
     // A bitstring's rescaling maximum and output bits, read while the tile before
     // its first one is worked on: reading the state on the spot put two global
     // latencies into every change of bitstring (n=61, d=32, 200 bitstrings: 3.90
@@ -819,8 +847,20 @@ __global__ void __launch_bounds__(SH::THREADS, SH::SMALL ? SMALL_CTAS_PER_SM : P
             if ((tid & 31u) == 0 && atomicExch(s_abort, 1) == 0) atomicAdd(p.fault, 1);
             break;
         }
+        bool idle = false;
+        if constexpr (SH::ZW) {
+            const uint32_t turn = (uint32_t)k & 7u, w = (tid >> 5) ^ turn;
+            sb = sb0 ^ (turn & 1u ? wslot[0] : 0u) ^ (turn & 2u ? wslot[1] : 0u) ^ (turn & 4u ? wslot[2] : 0u);
+            const uint32_t ti = tile_of_warp(p.skip.base, col, lane, (uint32_t)t << SH::CHL) ^ chunk_of_warp<SH>(col, w);
+            idle = __any_sync(0xffffffffu, ((uint32_t)__popc(ti & wout) + (uint32_t)__popc(w & wmask & 7u) + (wmask >> 3)) & 1u);
+        }
         if (t == 0 && tid == 0) p.exps[b * p.sstride + p.slot + 1] = cur_s;
 
+        if (idle) {
+            if (lane == 0) pbar_arrive(done0 + 8 * s);
+            if (++s == STAGES) { s = 0; ph ^= 1u; }
+            continue;
+        }
         float2* tile = stages + s * SH::ENTRIES;
         float2 P[16], Q[16];
         smem_read_j<SH, 0>(P, Q, tile, sb);
@@ -862,7 +902,11 @@ cudaError_t launch_shape(const PassParams& p, const CUtensorMap& m, int grid, cu
 
 template <int TYPE, int M>
 cudaError_t launch_one(const PassParams& p, const CUtensorMap& m, int grid, cudaStream_t st) {
-    return p.small ? launch_shape<Shape<TYPE, M, true>>(p, m, grid, st) : launch_shape<Shape<TYPE, M, false>>(p, m, grid, st);
+    if (p.small) return launch_shape<Shape<TYPE, M, true>>(p, m, grid, st);
+    if constexpr (warp_addr_bits(TYPE, M) > 0) {
+        if (p.warps.n > 0) return launch_shape<Shape<TYPE, M, false, true>>(p, m, grid, st);
+    }
+    return launch_shape<Shape<TYPE, M, false>>(p, m, grid, st);
 }
 
 #define TB_DEFINE_LAUNCH_PASS(TYPE, NAME)                                                      \

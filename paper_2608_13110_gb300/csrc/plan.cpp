@@ -380,6 +380,29 @@ public:
         return k;
     }
 
+    // Equations that tie the address bits [wlo, wlo + wn) of a tile's warp index to
+    // one another or to the bits C.. without [lo, lo + M) (index bits as in skip).
+    WarpSkip warps(int h, int C, int lo, int M, int wlo, int wn) const {
+        WarpSkip k;
+        std::memset(&k, 0, sizeof(k));
+        Support s = *this;
+        for (int b = 0; b < C; ++b)
+            if (b < wlo || b >= wlo + wn) s.eliminate(b);
+        for (int b = lo; b < lo + M; ++b) s.eliminate(b);
+        const uint64_t low = ((uint64_t)1 << (lo - C)) - 1;
+        for (int b = wlo; b < wlo + wn; ++b)  // one equation per warp bit at most: take it out with the bit
+            for (int i = 0; i < s.n_; ++i)
+                if (s.eq_[i].mask >> b & 1) {
+                    const Eq e = s.eq_[i];
+                    k.out[k.n] = (uint32_t)((e.mask >> C & low) | (e.mask >> (lo + M) << (lo - C)));
+                    k.warp[k.n] = (uint32_t)(e.mask >> wlo & ((1u << wn) - 1u)) | ((uint32_t)e.value << 3);
+                    ++k.n;
+                    s.eliminate(b);
+                    break;
+                }
+        return k;
+    }
+
     // The equation that determines bit var from the higher bits, if any (after the
     // lower bits have been eliminated): parity(address & *mask) ^ *value.
     bool determined(int var, uint64_t* mask, int* value) const {
@@ -430,6 +453,8 @@ static void tile_skips(Plan& P, Support s) {
         // outside the chunks; at least one tile of visited ones
         d.skip = bottom_type(d.type) ? s.skip(h, bot_chunk_bits(d.M), -1, 0, h - TILE_BITS)
                                      : s.skip(h, high_low_bits(d.M), d.lo, d.M, h - TILE_BITS);
+        const int wn = warp_addr_bits(d.type, d.M);
+        if (wn && h <= MAX_H) d.warps = s.warps(h, high_low_bits(d.M), d.lo, d.M, warp_low_bit(d.M), wn);
     }
     for (TcPass& d : P.tc_passes) {  // outside the window and the TC_VEC_BITS lowest other bits
         advance(d.step0);

@@ -187,6 +187,19 @@ __host__ __device__ constexpr int small_row_log2(int type, int M) {
 }
 __host__ __device__ constexpr bool has_small_tiles(int type, int M) { return bottom_type(type) || M <= 9; }
 
+// Zero warps of a pass whose tiles hold low address bits in the warp index
+// (8- and 9-bit windows above bit 0): warp w of tile t holds something only if
+// parity(t & out[i]) ^ parity(w & (warp[i] & 7)) = warp[i] >> 3 for every i < n.
+struct WarpSkip {
+    int n;
+    uint32_t out[3], warp[3];
+};
+// Lowest address bit and number of address bits in the warp index (0: none).
+__host__ __device__ constexpr int warp_low_bit(int M) { return M == 9 ? 1 : 2; }
+__host__ __device__ constexpr int warp_addr_bits(int type, int M) {
+    return bottom_type(type) ? 0 : M == 9 ? 3 : M == 8 ? 2 : 0;
+}
+
 // Rows of a late crossing of an open plan: output rows visited, and which of
 // the input rows 2r', 2r'+1 may be nonzero (one: both == 0, the row whose low
 // bit is parity(r' & mask) ^ fix). The others are not read or written.
@@ -207,6 +220,7 @@ struct PassDesc {
     int xs_step[2];  // bit of the pass's variant mask set by an output bit, -1 if none
     int xs_q[2];     // the qubit whose output bit sets it
     TileSkip skip;   // tiles visited
+    WarpSkip warps;  // and the warps of those with something to do
 };
 
 // ---- Tensor-core dense blocks (TB_PRECISION_TF32X3 / TB_PRECISION_BF16X3) --

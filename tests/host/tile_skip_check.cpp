@@ -93,6 +93,18 @@ int main(int argc, char** argv) {
         if (!bottom)
             for (int b = 0; b < p.M; ++b) tile.push_back(p.lo + b);
         if (!check(p.step0, tile, p.skip)) return 2;
+        // warps with nothing to do: the entries with these low address bits are zero
+        const int wn = warp_addr_bits(p.type, p.M);
+        for (size_t i = 0; i < B.size() && wn; ++i) {
+            if (B[i] == 0.0) continue;
+            const uint32_t w = (uint32_t)(i >> warp_low_bit(p.M)) & ((1u << wn) - 1u);
+            const uint32_t t = (uint32_t)((i >> 4 & (((size_t)1 << (p.lo - 4)) - 1)) | (i >> (p.lo + p.M) << (p.lo - 4)));
+            for (int e = 0; e < p.warps.n; ++e)
+                if ((__builtin_parity(t & p.warps.out[e]) ^ __builtin_parity(w & p.warps.warp[e] & 7u)) != (int)(p.warps.warp[e] >> 3)) {
+                    printf("pass at step %d: warp %u leaves out entry %zu, which is not zero\n", p.step0, w, i);
+                    return 2;
+                }
+        }
         if (p.skip.n > h - TILE_BITS) {
             printf("pass at step %d visits less than one tile\n", p.step0);
             return 2;
