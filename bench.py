@@ -187,9 +187,9 @@ def kernel_code_hash() -> str:
     return hashlib.sha256(src.encode()).hexdigest()[:16]
 
 
-def pass_traffic(h: int):
-    """DRAM bytes per pass launch from the committed ncu summary, scaled to a
-    2^h boundary, or None if absent or taken on other kernel sources."""
+def pass_traffic(entries: float):
+    """DRAM bytes per pass launch from the committed ncu summary, scaled to the
+    entries a pass visits, or None if absent or taken on other kernel sources."""
     path = os.path.join(ROOT, "profiles", "pass_kernel_traffic.txt")
     if not os.path.exists(path):
         return None
@@ -202,7 +202,7 @@ def pass_traffic(h: int):
     if kv.get("pass_kernel_code_sha256_16") != digest:
         return None
     try:
-        return float(kv["dram_bytes_per_entry"]) * float(2 ** h)
+        return float(kv["dram_bytes_per_entry"]) * entries
     except (KeyError, ValueError):
         return None
 
@@ -320,7 +320,9 @@ def run_ours(args, rank, world, local):
     p = prof["pass"]
     achieved = p["bytes"] / (p["ms"] / 1e3) / 1e9 if p["ms"] > 0 else None
     n_launch = sum(v["launches"] for v in prof.values())
-    traffic = pass_traffic(h) if args.precision == "fp32" else None
+    # entries of the tiles a pass visits (tiles known to be zero are left out), mean per launch
+    entries = p["bytes"] / 16.0 / max(1, p["launches"])
+    traffic = pass_traffic(entries) if args.precision == "fp32" else None
 
     line = {
         "metric": metric, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
@@ -343,7 +345,8 @@ def run_ours(args, rank, world, local):
                    "would need for the same amps/s (secondary, not a measured bandwidth)"},
         "roofline": {"bound": "hbm", "achieved": achieved, "peak": hbm_peak, "unit": "GB/s",
                      "frac": (achieved / hbm_peak) if achieved else None, "traffic": traffic,
-                     "traffic_over_algorithmic": (traffic / (16.0 * 2.0 ** h)) if traffic else None,
+                     "traffic_over_algorithmic": (traffic / (16.0 * entries)) if traffic else None,
+                     "entries_visited": p["bytes"] / 16.0 / max(1.0, 2.0 ** h * nb * args.steps * info["n_passes"]),
                      "kernel": "pass_kernel" if args.precision == "fp32" else "tc_pass_kernel",
                      "peak_source": f"{peak_src} copy bandwidth",
                      "pass_launches": p["launches"], "pass_ms_total": p["ms"],
@@ -361,17 +364,18 @@ def run_ours(args, rank, world, local):
 
 def fma_pipe_fraction(args, info, nb, h, p, clk, dev):
     """The FP32 passes' other ceiling: the multiply-adds the pass kernels
-    spend per entry (8 per paired step, 16 per row turn's 4x4 block: the
-    plan's pass_madds), over the pass kernels' measured time, against SMs x
-    128 FP32 lanes x the SM clock (one FMA per lane and cycle; the paired FFMA2
-    issues two lanes' worth in two cycles). Secondary to the HBM roofline: the
-    two floors are within 15 % of each other at width 32."""
+    spend per entry (8 per paired step, 16 per row turn's 4x4 block: the mean
+    of the plan's pass_madds over its passes), for the entries they visit, over
+    the pass kernels' measured time, against SMs x 128 FP32 lanes x the SM clock
+    (one FMA per lane and cycle; the paired FFMA2 issues two lanes' worth in two
+    cycles). Secondary to the HBM roofline: the two floors are within 15 % of
+    each other at width 32."""
     if args.precision != "fp32" or p["ms"] <= 0:
         return None
     import torch
     sms = torch.cuda.get_device_properties(dev).multi_processor_count
     mhz = clk.get("sm_max_mhz") or 2070.0
-    fma = float(nb) * args.steps * info["pass_madds"] * 2.0 ** h
+    fma = p["bytes"] / 16.0 * info["pass_madds"] / max(1, info["n_passes"])
     achieved = fma / (p["ms"] / 1e3) / 1e12
     peak = sms * 128 * mhz * 1e6 / 1e12
     return {"achieved": achieved, "peak": peak, "unit": "TFMA/s", "frac": achieved / peak,
