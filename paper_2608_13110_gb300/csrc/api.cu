@@ -238,15 +238,16 @@ bool small_tiles(const PassDesc& d, int64_t ntiles, int nsm) {
 // 8: 44.2 -> 44.5.
 bool pass_runs(int tile_shift, int grid) { return ((int64_t)1 << tile_shift) < 8 * (int64_t)grid; }
 
-cudaError_t launch_pass(const PassDesc& d, const PassParams& p, const CUtensorMap& m, int grid, cudaStream_t st) {
+cudaError_t launch_pass(const PassDesc& d, const PassParams& p, const StepG* host_steps, const CUtensorMap& m, int grid,
+                        cudaStream_t st) {
     switch (d.type) {
-        case P_FWD: return launch_pass_t0(d.M, p, m, grid, st);
-        case P_REV: return launch_pass_t1(d.M, p, m, grid, st);
-        case P_TOP: return launch_pass_t2(d.M, p, m, grid, st);
-        case P_BOT: return launch_pass_t3(d.M, p, m, grid, st);
-        case P_BOT_START: return launch_pass_t4(d.M, p, m, grid, st);
-        case P_BOT_END: return launch_pass_t5(d.M, p, m, grid, st);
-        case P_TOP_END: return launch_pass_t6(d.M, p, m, grid, st);
+        case P_FWD: return launch_pass_t0(d.M, p, host_steps, m, grid, st);
+        case P_REV: return launch_pass_t1(d.M, p, host_steps, m, grid, st);
+        case P_TOP: return launch_pass_t2(d.M, p, host_steps, m, grid, st);
+        case P_BOT: return launch_pass_t3(d.M, p, host_steps, m, grid, st);
+        case P_BOT_START: return launch_pass_t4(d.M, p, host_steps, m, grid, st);
+        case P_BOT_END: return launch_pass_t5(d.M, p, host_steps, m, grid, st);
+        case P_TOP_END: return launch_pass_t6(d.M, p, host_steps, m, grid, st);
         default: return cudaErrorInvalidValue;
     }
 }
@@ -387,7 +388,7 @@ int run_device(const Plan& P, const uint8_t* d_bits, int64_t nb, void* d_ws, int
             const int grid = pp.small ? (int)pp.ntiles : (int)std::min<int64_t>(pp.ntiles, (int64_t)PASS_CTAS_PER_SM * nsm);
             pp.runs = pass_runs(pp.tile_shift, grid) ? 1 : 0;
             ProfScope ps(PC_PASS, 16.0 * (double)nbat * (double)(b_stride >> d.skip.n), st);
-            TB_CUDA(launch_pass(d, pp, tmap, grid, st));
+            TB_CUDA(launch_pass(d, pp, P.pass_steps.data() + d.pstep0, tmap, grid, st));
         }
 
         if (P.open_k) {  // Algorithm 2: join, late crossings, FP64 output

@@ -5,32 +5,41 @@
 // every step of one window of address bits is applied in a single read + write
 // of the boundary.
 //
-// A pass applies a compile-time sequence of controlled 2x2 steps to every
-// tile of 2^13 complex64 entries: the window's M address bits plus 13-M low
-// address bits (the 13 lowest bits when the window starts at bit 0). At a row
-// turn the four steps on the window's two outermost bits run as one 4x4 block
-// (composed on the host, see tb_internal.h).
+// A pass applies a compile-time sequence of controlled 2x2 steps to tiles of
+// 2^13 complex64 entries: the window's M address bits in chunks that the
+// copies want (see pass_chunk_log2). Chunks that are exactly zero are not
+// visited (TileSkip). At a row turn the four steps on the window's two
+// outermost bits run as one 4x4 block (composed on the host, see tb_internal.h).
 //
 // Warp-specialised, one persistent CTA per SM:
-//   * one producer thread moves whole tiles between HBM and a 3-stage ring of
-//     shared-memory stages with tensor copies (cp.async.bulk.tensor, 128-byte
-//     swizzle; 64-byte rows and swizzle for 10-bit windows above bit 0): a
-//     load completes on the stage's "full" mbarrier; once the
-//     consumers have written the stage back it is stored in place with one
-//     bulk tensor store, and as soon as the store has read the stage the next
-//     tile's load is issued into it;
-//   * 8 consumer warps never touch global memory and never wait for one
-//     another: warp w owns the 1024 entries of the tile that share 3 "warp
-//     bits" and holds them as 32 entries per thread: 5 address bits in
-//     registers, 5 on the lanes. Every window bit is one of these 10, so a
-//     step on a register bit is register arithmetic and a step on a lane bit
-//     exchanges the partner lane's entries with warp shuffles. A warp reads
-//     its entries from the stage once, applies every step, writes them back
-//     and arrives on the stage's "done" mbarrier. HBM traffic, shared-memory
+//   * one producer warp moves whole tiles between HBM and a 3-stage ring of
+//     shared-memory stages with tensor copies (cp.async.bulk.tensor, one per
+//     chunk, 128-byte swizzle; 64-byte rows and swizzle for 10-bit windows
+//     above bit 0): a load completes on the stage's "full" mbarrier; once the
+//     consumers have written the stage back it is stored in place, and as soon
+//     as the stores have read the stage the next tile's loads are issued into it;
+//   * 8 consumer warps read global memory only for a bitstring's state, a tile
+//     ahead, and never wait for one another: warp w owns the 1024 entries of the
+//     tile that share 3 "warp bits" and holds them as 32 entries per thread: 5
+//     address bits in registers, 5 on the lanes. Every window bit is one of
+//     these 10, so a step on a register bit is register arithmetic and a step on
+//     a lane bit exchanges the partner lane's entries with warp shuffles. A warp
+//     reads its entries from the stage once, applies every step, writes them
+//     back and arrives on the stage's "done" mbarrier. HBM traffic, shared-memory
 //     traffic and the arithmetic of different warps all overlap.
 // The tensor map orders the tile's address bits so that every warp access to
 // a stage is free of shared-memory bank conflicts, except in the 64-byte-row
-// layout, where they are two-way (see slot_of).
+// layout of 10-bit windows, where they are two-way (see slot_of).
+//
+// What bounds it: HBM and the FP32 pipe about equally. The consumer loop alone
+// (no copies) takes, in cycles per tile, 5620 for a 9-bit forward window, 6100
+// reversed, 7320 for a 7-bit top turn and 13120 for a 10-bit bottom turn; the
+// measured HBM copy rate allows a tile every 6050. A paired FMA whose three
+// operands are all fresh registers takes 3 issue cycles instead of 2 (see
+// step_uniform) and two warps share a scheduler, which is why the loop reaches
+// 0.65 to 0.75 of the FMA rate. n=70, d=64 (width 32), 16 bitstrings: 0.36
+// amplitudes/s visiting every tile, 1.33 leaving the zeros out (27 % of the entries
+// visited; 0.75 of the HBM copy rate and 0.63 of the FMA rate on those).
 //
 // Rescaling: the producer of this pass's input left max(|re|,|im|) of its
 // output in maxs[slot]; this pass multiplies its input by 2^s (exact; folded
@@ -236,7 +245,7 @@ constexpr int VBIT = 4;
 constexpr int KIND_F = 0, KIND_VC = 1, KIND_VT = 2, KIND_L = 3, KIND_BL = 4, KIND_BV = 5;
 constexpr int CO = 48;  // packed coefficients per (step, variant)
 
-__device__ __forceinline__ float2 f2x(float a) { return make_float2(a, a); }
+__host__ __device__ __forceinline__ float2 f2x(float a) { return make_float2(a, a); }
 __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
 __device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
 __device__ __forceinline__ float2 swap2(float2 a) { return make_float2(a.y, a.x); }
@@ -262,39 +271,41 @@ __device__ __forceinline__ void load_cf(float2 (&c)[N], const float2* src, float
 
 // Register target bit K < 4 (pairs of packed registers). CK: -1 none (block
 // 0), 0..3 control register bit (block per pair), 4 control = register bit 4
-// (lane-split block), 5 control on a lane (block chosen by the caller).
+// (lane-split block), 5 control on a lane (block chosen by the caller). The
+// pairs of one control value together: half the coefficients live at a time
+// (9-bit top turn 11980 cycles per tile in the registers' order, 10360 so).
 template <int K, int CK>
-__device__ __forceinline__ void step_pairs(float2 (&P)[16], float2 (&Q)[16], const float2 (&c0)[12],
-                                           const float2 (&c1)[12]) {
+__device__ __forceinline__ void step_pairs(float2 (&P)[16], float2 (&Q)[16], const float2* c0, const float2* c1) {
+    constexpr bool split = CK >= 0 && CK < 4;
 #pragma unroll
-    for (int k = 0; k < 16; ++k) {
-        if (k & (1 << K)) continue;
-        const int k1 = k | (1 << K);
-        const bool hi = (CK >= 0 && CK < 4) ? (((k >> CK) & 1) != 0) : false;
-        float2 p0, q0, p1, q1;
-        if (hi) {
-            cmac_planar(c1, P[k], Q[k], P[k1], Q[k1], p0, q0);
-            cmac_planar(c1 + 6, P[k], Q[k], P[k1], Q[k1], p1, q1);
-        } else {
-            cmac_planar(c0, P[k], Q[k], P[k1], Q[k1], p0, q0);
-            cmac_planar(c0 + 6, P[k], Q[k], P[k1], Q[k1], p1, q1);
+    for (int hv = 0; hv < (split ? 2 : 1); ++hv) {
+        const float2* c = hv ? c1 : c0;
+#pragma unroll
+        for (int k = 0; k < 16; ++k) {
+            if (k & (1 << K)) continue;
+            if (split && ((k >> (CK & 3)) & 1) != hv) continue;
+            const int k1 = k | (1 << K);
+            float2 p0, q0, p1, q1;
+            cmac_planar(c, P[k], Q[k], P[k1], Q[k1], p0, q0);
+            cmac_planar(c + 6, P[k], Q[k], P[k1], Q[k1], p1, q1);
+            P[k] = p0; Q[k] = q0; P[k1] = p1; Q[k1] = q1;
         }
-        P[k] = p0; Q[k] = q0; P[k1] = p1; Q[k1] = q1;
     }
 }
 
 // Register target bit 4: the pair is the two halves of one packed register.
 template <int CK>
-__device__ __forceinline__ void step_halves(float2 (&P)[16], float2 (&Q)[16], const float2 (&c0)[12],
-                                            const float2 (&c1)[12]) {
+__device__ __forceinline__ void step_halves(float2 (&P)[16], float2 (&Q)[16], const float2* c0, const float2* c1) {
+    constexpr bool split = CK >= 0 && CK < 4;
 #pragma unroll
-    for (int k = 0; k < 16; ++k) {
-        const bool hi = (CK >= 0 && CK < 4) ? (((k >> CK) & 1) != 0) : false;
-        const float2 p = P[k], q = Q[k];
-        float2 op, oq;
-        if (hi) cmac_planar(c1, p, q, swap2(p), swap2(q), op, oq);  // [Ar Ai -Ai Br Bi -Bi]
-        else    cmac_planar(c0, p, q, swap2(p), swap2(q), op, oq);
-        P[k] = op; Q[k] = oq;
+    for (int hv = 0; hv < (split ? 2 : 1); ++hv) {
+        const float2* c = hv ? c1 : c0;
+#pragma unroll
+        for (int k = 0; k < 16; ++k) {
+            if (split && ((k >> (CK & 3)) & 1) != hv) continue;
+            const float2 p = P[k], q = Q[k];
+            cmac_planar(c, p, q, swap2(p), swap2(q), P[k], Q[k]);
+        }
     }
 }
 
@@ -376,12 +387,82 @@ __host__ __device__ constexpr int step_kind(int i) {
     return KIND_F;
 }
 
+// Steps whose coefficients come from the kernel's parameters instead of shared
+// memory: steps on a register bit that no lane bit controls and no output bit
+// changes, so that they are the same for every thread and bitstring. A paired
+// FMA takes 3.0 issue cycles with three fresh register pairs and 2.1 with the
+// coefficient in the constant bank (a coefficient that several FMAs in a row
+// share: 2.2, but no order of the steps' FMAs made ptxas keep it). Consumer loop
+// alone, cycles per tile: 9-bit forward window 6030 -> 5620, reversed 6510 -> 6100,
+// 7-bit top turn 7900 -> 7320, 9-bit top turn 11150 -> 10360, 8-bit window forward
+// 5300 -> 4860, 10-bit bottom turn 13150 -> 13120 (its lane steps and block
+// dominate). n=28, d=42, dense gates, 32 bitstrings: 6.00 -> 5.78 ms; n=70, d=56,
+// two bitstrings: 131.8 -> 128.2 ms.
+// Not the first step, which carries the rescale; small tiles have one tile per
+// CTA, where the time is set-up and latency (367 and 361 us on n=33, d=35, no
+// difference between runs), and smaller parameters launch faster.
+template <class SH>
+__host__ __device__ constexpr bool step_uniform(int i) {
+    if (SH::SMALL || i == 0 || i == SH::BLK || output_step(SH::TYPE, SH::M, i)) return false;
+    return SH::regpos(SH::tgt(i)) >= 0 && (SH::ctl(i) < 0 || SH::regpos(SH::ctl(i)) >= 0);
+}
+template <class SH>
+__host__ __device__ constexpr int uniform_index(int n) {  // uniform steps before step n
+    int u = 0;
+    for (int i = 0; i < n; ++i) u += step_uniform<SH>(i) ? 1 : 0;
+    return u;
+}
+constexpr int UCO = 24;  // their packed coefficients
+template <class SH>
+struct PassConst {
+    float2 c[uniform_index<SH>(SH::NS) > 0 ? uniform_index<SH>(SH::NS) : 1][UCO];
+};
+
 template <class SH>
 __host__ __device__ constexpr uint64_t step_kinds() {
     uint64_t k = 0;
     static_assert(3 * SH::NS <= 64, "three kind bits per step");
     for (int i = 0; i < SH::NS; ++i) k |= (uint64_t)step_kind<SH>(i) << (3 * i);
     return k;
+}
+
+template <class SH>
+__host__ __device__ constexpr uint32_t uniform_mask() {
+    uint32_t m = 0;
+    for (int i = 0; i < SH::NS; ++i) m |= (step_uniform<SH>(i) ? 1u : 0u) << i;
+    return m;
+}
+
+// The packed coefficients of a step on a register bit (KIND_F, _VC, _VT) from
+// its blocks g[c*4 + a'*2 + s].
+__host__ __device__ inline void pack_register_step(int kind, const float2* g, float2* o) {
+    if (kind == KIND_F) {
+        for (int c = 0; c < 2; ++c)
+            for (int e = 0; e < 4; ++e) {
+                const float2 z = g[c * 4 + e];
+                o[c * 12 + 3 * e + 0] = f2x(z.x);
+                o[c * 12 + 3 * e + 1] = f2x(z.y);
+                o[c * 12 + 3 * e + 2] = f2x(-z.y);
+            }
+    } else if (kind == KIND_VC) {
+        for (int e = 0; e < 4; ++e) {
+            const float2 z0 = g[e], z1 = g[4 + e];
+            o[3 * e + 0] = make_float2(z0.x, z1.x);
+            o[3 * e + 1] = make_float2(z0.y, z1.y);
+            o[3 * e + 2] = make_float2(-z0.y, -z1.y);
+        }
+    } else if (kind == KIND_VT) {
+        for (int c = 0; c < 2; ++c) {
+            const float2 A0 = g[c * 4 + 0], A1 = g[c * 4 + 3];  // own half: g00 (lo), g11 (hi)
+            const float2 B0 = g[c * 4 + 1], B1 = g[c * 4 + 2];  // other half: g01 (lo), g10 (hi)
+            o[c * 12 + 0] = make_float2(A0.x, A1.x);
+            o[c * 12 + 1] = make_float2(A0.y, A1.y);
+            o[c * 12 + 2] = make_float2(-A0.y, -A1.y);
+            o[c * 12 + 3] = make_float2(B0.x, B1.x);
+            o[c * 12 + 4] = make_float2(B0.y, B1.y);
+            o[c * 12 + 5] = make_float2(-B0.y, -B1.y);
+        }
+    }
 }
 
 // Stage the packed coefficients of every step and variant into shared memory.
@@ -398,8 +479,10 @@ __host__ __device__ constexpr uint64_t step_kinds() {
 template <class SH>
 __device__ __forceinline__ void stage_coefficients(const StepG* steps, float2* sc, uint32_t tid) {
     constexpr uint64_t KINDS = step_kinds<SH>();
+    constexpr uint32_t UNIFORM = uniform_mask<SH>();
     for (int w = tid; w < SH::NB; w += SH::THREADS) {
         const int i = w < 2 * SH::NS ? w >> 1 : SH::XM, x = w & 1;
+        if ((UNIFORM >> i) & 1u) continue;
         float2* o = sc + w * CO;
         for (int e = 0; e < CO; ++e) o[e] = make_float2(0.f, 0.f);
         const int kind = (int)((KINDS >> (3 * i)) & 7u);
@@ -430,32 +513,8 @@ __device__ __forceinline__ void stage_coefficients(const StepG* steps, float2* s
             continue;
         }
         const float2* g = steps[pass_entry(SH::TYPE, SH::M, i)].g[x];  // [c*4 + a'*2 + s]
-        if (kind == KIND_F) {
-            for (int c = 0; c < 2; ++c)
-                for (int e = 0; e < 4; ++e) {
-                    const float2 z = g[c * 4 + e];
-                    o[c * 12 + 3 * e + 0] = f2x(z.x);
-                    o[c * 12 + 3 * e + 1] = f2x(z.y);
-                    o[c * 12 + 3 * e + 2] = f2x(-z.y);
-                }
-        } else if (kind == KIND_VC) {
-            for (int e = 0; e < 4; ++e) {
-                const float2 z0 = g[e], z1 = g[4 + e];
-                o[3 * e + 0] = make_float2(z0.x, z1.x);
-                o[3 * e + 1] = make_float2(z0.y, z1.y);
-                o[3 * e + 2] = make_float2(-z0.y, -z1.y);
-            }
-        } else if (kind == KIND_VT) {
-            for (int c = 0; c < 2; ++c) {
-                const float2 A0 = g[c * 4 + 0], A1 = g[c * 4 + 3];  // own half: g00 (lo), g11 (hi)
-                const float2 B0 = g[c * 4 + 1], B1 = g[c * 4 + 2];  // other half: g01 (lo), g10 (hi)
-                o[c * 12 + 0] = make_float2(A0.x, A1.x);
-                o[c * 12 + 1] = make_float2(A0.y, A1.y);
-                o[c * 12 + 2] = make_float2(-A0.y, -A1.y);
-                o[c * 12 + 3] = make_float2(B0.x, B1.x);
-                o[c * 12 + 4] = make_float2(B0.y, B1.y);
-                o[c * 12 + 5] = make_float2(-B0.y, -B1.y);
-            }
+        if (kind != KIND_L) {
+            pack_register_step(kind, g, o);
         } else {
             for (int a = 0; a < 2; ++a) {
                 float2* oa = o + 24 * a;
@@ -497,7 +556,7 @@ __device__ __forceinline__ void smem_write_j(const float2 (&P)[16], const float2
 
 template <class SH, int I>
 __device__ __forceinline__ void apply_step(float2 (&P)[16], float2 (&Q)[16], const float2* sc,
-                                           uint32_t xmask, float scale, uint32_t tid) {
+                                           const PassConst<SH>& pc, uint32_t xmask, float scale, uint32_t tid) {
     constexpr int T = SH::tgt(I), CB = SH::ctl(I);
     constexpr int kind = step_kind<SH>(I);
     // control: -1 none, 0..4 register bit, 5 on a lane (the same for all of
@@ -534,6 +593,10 @@ __device__ __forceinline__ void apply_step(float2 (&P)[16], float2 (&Q)[16], con
             if constexpr (CK >= 0) load_cf(c1, ca + 6, s);
         }
         step_lane<(CK == 4 || CK == 5) ? -1 : CK>(P, Q, c0, c1, 1 << L);
+    } else if constexpr (step_uniform<SH>(I)) {
+        const float2* c = pc.c[uniform_index<SH>(I)];
+        if constexpr (kind == KIND_VT) step_halves<CK>(P, Q, c, c + 12);
+        else step_pairs<SH::regpos(T), CK>(P, Q, c, c + 12);
     } else {
         constexpr int K = SH::regpos(T);
         float2 c0[12], c1[12];
@@ -552,11 +615,11 @@ __device__ __forceinline__ void apply_step(float2 (&P)[16], float2 (&Q)[16], con
 }
 
 template <class SH, int I>
-__device__ __forceinline__ void run_steps(float2 (&P)[16], float2 (&Q)[16], const float2* sc, uint32_t xmask,
-                                          float scale, uint32_t tid) {
+__device__ __forceinline__ void run_steps(float2 (&P)[16], float2 (&Q)[16], const float2* sc,
+                                          const PassConst<SH>& pc, uint32_t xmask, float scale, uint32_t tid) {
     if constexpr (I < SH::NS) {
-        apply_step<SH, I>(P, Q, sc, xmask, scale, tid);
-        run_steps<SH, I + 1>(P, Q, sc, xmask, scale, tid);
+        apply_step<SH, I>(P, Q, sc, pc, xmask, scale, tid);
+        run_steps<SH, I + 1>(P, Q, sc, pc, xmask, scale, tid);
     }
 }
 
@@ -668,7 +731,8 @@ constexpr int pass_smem_bytes() {
 
 template <class SH>
 __global__ void __launch_bounds__(SH::THREADS, SH::SMALL ? SMALL_CTAS_PER_SM : PASS_CTAS_PER_SM)
-    pass_kernel(const __grid_constant__ PassParams p, const __grid_constant__ CUtensorMap tmap) {
+    pass_kernel(const __grid_constant__ PassParams p, const __grid_constant__ CUtensorMap tmap,
+                const __grid_constant__ PassConst<SH> pc) {
     static_assert(SH::valid(), "invalid pass shape");
     static_assert(SH::NS <= XM_HIGH_BIT, "variant mask: one bit per step, bit XM_HIGH_BIT for the four-variant step");
     constexpr int STAGES = SH::STAGES;
@@ -864,7 +928,7 @@ __global__ void __launch_bounds__(SH::THREADS, SH::SMALL ? SMALL_CTAS_PER_SM : P
         float2* tile = stages + s * SH::ENTRIES;
         float2 P[16], Q[16];
         smem_read_j<SH, 0>(P, Q, tile, sb);
-        run_steps<SH, 0>(P, Q, sc, xmask, scale, tid);
+        run_steps<SH, 0>(P, Q, sc, pc, xmask, scale, tid);
 #pragma unroll
         for (int j = 0; j < 16; ++j)
             runmax = fmaxf(runmax, fmaxf(fmaxf(fabsf(P[j].x), fabsf(P[j].y)), fmaxf(fabsf(Q[j].x), fabsf(Q[j].y))));
@@ -878,17 +942,27 @@ __global__ void __launch_bounds__(SH::THREADS, SH::SMALL ? SMALL_CTAS_PER_SM : P
     if (!one_tile) grid_release();
 }
 
-// Launchers, one translation unit per pass type (pass_t<type>.cu).
-cudaError_t launch_pass_t0(int M, const PassParams& p, const CUtensorMap& m, int grid, cudaStream_t st);
-cudaError_t launch_pass_t1(int M, const PassParams& p, const CUtensorMap& m, int grid, cudaStream_t st);
-cudaError_t launch_pass_t2(int M, const PassParams& p, const CUtensorMap& m, int grid, cudaStream_t st);
-cudaError_t launch_pass_t3(int M, const PassParams& p, const CUtensorMap& m, int grid, cudaStream_t st);
-cudaError_t launch_pass_t4(int M, const PassParams& p, const CUtensorMap& m, int grid, cudaStream_t st);
-cudaError_t launch_pass_t5(int M, const PassParams& p, const CUtensorMap& m, int grid, cudaStream_t st);
-cudaError_t launch_pass_t6(int M, const PassParams& p, const CUtensorMap& m, int grid, cudaStream_t st);
+// Launchers, one translation unit per pass type (pass_t<type>.cu). host_steps:
+// the pass's entries of the pass-step table in host memory (p.steps is its copy
+// on the device).
+cudaError_t launch_pass_t0(int M, const PassParams& p, const StepG* host_steps, const CUtensorMap& m, int grid,
+                           cudaStream_t st);
+cudaError_t launch_pass_t1(int M, const PassParams& p, const StepG* host_steps, const CUtensorMap& m, int grid,
+                           cudaStream_t st);
+cudaError_t launch_pass_t2(int M, const PassParams& p, const StepG* host_steps, const CUtensorMap& m, int grid,
+                           cudaStream_t st);
+cudaError_t launch_pass_t3(int M, const PassParams& p, const StepG* host_steps, const CUtensorMap& m, int grid,
+                           cudaStream_t st);
+cudaError_t launch_pass_t4(int M, const PassParams& p, const StepG* host_steps, const CUtensorMap& m, int grid,
+                           cudaStream_t st);
+cudaError_t launch_pass_t5(int M, const PassParams& p, const StepG* host_steps, const CUtensorMap& m, int grid,
+                           cudaStream_t st);
+cudaError_t launch_pass_t6(int M, const PassParams& p, const StepG* host_steps, const CUtensorMap& m, int grid,
+                           cudaStream_t st);
 
 template <class SH>
-cudaError_t launch_shape(const PassParams& p, const CUtensorMap& m, int grid, cudaStream_t st) {
+cudaError_t launch_shape(const PassParams& p, const StepG* host_steps, const CUtensorMap& m, int grid,
+                         cudaStream_t st) {
     if constexpr (!SH::valid()) {
         return cudaErrorInvalidValue;
     } else {
@@ -896,28 +970,36 @@ cudaError_t launch_shape(const PassParams& p, const CUtensorMap& m, int grid, cu
         static_assert(smem <= 227 * 1024, "pass kernel shared memory");
         cudaError_t e = cudaFuncSetAttribute(pass_kernel<SH>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         if (e != cudaSuccess) return e;
-        return launch_after(pass_kernel<SH>, grid, SH::THREADS, smem, st, p, m);
+        PassConst<SH> pc{};
+        for (int i = 0; i < SH::NS; ++i) {
+            if (!step_uniform<SH>(i)) continue;
+            if (p.xs_step0 == i || p.xs_step1 == i) return cudaErrorInvalidValue;  // output_step excludes it
+            pack_register_step(step_kind<SH>(i), host_steps[pass_entry(SH::TYPE, SH::M, i)].g[0],
+                               pc.c[uniform_index<SH>(i)]);
+        }
+        return launch_after(pass_kernel<SH>, grid, SH::THREADS, smem, st, p, m, pc);
     }
 }
 
 template <int TYPE, int M>
-cudaError_t launch_one(const PassParams& p, const CUtensorMap& m, int grid, cudaStream_t st) {
-    if (p.small) return launch_shape<Shape<TYPE, M, true>>(p, m, grid, st);
+cudaError_t launch_one(const PassParams& p, const StepG* host_steps, const CUtensorMap& m, int grid, cudaStream_t st) {
+    if (p.small) return launch_shape<Shape<TYPE, M, true>>(p, host_steps, m, grid, st);
     if constexpr (warp_addr_bits(TYPE, M) > 0) {
-        if (p.warps.n > 0) return launch_shape<Shape<TYPE, M, false, true>>(p, m, grid, st);
+        if (p.warps.n > 0) return launch_shape<Shape<TYPE, M, false, true>>(p, host_steps, m, grid, st);
     }
-    return launch_shape<Shape<TYPE, M, false>>(p, m, grid, st);
+    return launch_shape<Shape<TYPE, M, false>>(p, host_steps, m, grid, st);
 }
 
 #define TB_DEFINE_LAUNCH_PASS(TYPE, NAME)                                                      \
-    cudaError_t NAME(int M, const PassParams& p, const CUtensorMap& m, int grid, cudaStream_t st) { \
+    cudaError_t NAME(int M, const PassParams& p, const StepG* host_steps, const CUtensorMap& m, int grid,  \
+                     cudaStream_t st) {                                                   \
         switch (M) {                                                                          \
-            case 5: return launch_one<TYPE, 5>(p, m, grid, st);                               \
-            case 6: return launch_one<TYPE, 6>(p, m, grid, st);                               \
-            case 7: return launch_one<TYPE, 7>(p, m, grid, st);                               \
-            case 8: return launch_one<TYPE, 8>(p, m, grid, st);                               \
-            case 9: return launch_one<TYPE, 9>(p, m, grid, st);                               \
-            case 10: return launch_one<TYPE, 10>(p, m, grid, st);                             \
+            case 5: return launch_one<TYPE, 5>(p, host_steps, m, grid, st);               \
+            case 6: return launch_one<TYPE, 6>(p, host_steps, m, grid, st);               \
+            case 7: return launch_one<TYPE, 7>(p, host_steps, m, grid, st);               \
+            case 8: return launch_one<TYPE, 8>(p, host_steps, m, grid, st);               \
+            case 9: return launch_one<TYPE, 9>(p, host_steps, m, grid, st);               \
+            case 10: return launch_one<TYPE, 10>(p, host_steps, m, grid, st);             \
             default: return cudaErrorInvalidValue;                                            \
         }                                                                                     \
     }

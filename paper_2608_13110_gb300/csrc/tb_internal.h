@@ -87,6 +87,12 @@ __host__ __device__ constexpr int pass_blk(int type, int M) {
 __host__ __device__ constexpr int pass_xm(int type, int M) { return type == P_TOP ? M - 3 : -1; }
 constexpr int XM_HIGH_BIT = 31;
 
+// Whether an output bit may change step i: those steps create the value above
+// the boundary's last address bit, the window's last bit in TOP and TOP_END passes.
+__host__ __device__ constexpr bool output_step(int type, int M, int i) {
+    return i == pass_xm(type, M) || (type == P_TOP_END && i == pass_nsteps(type, M) - 1);
+}
+
 // A turn block in the pass-step table: BLK_ENTRIES consecutive StepG read as
 // float2[4 variants][2 control values][4 rows q'][4 columns q], block index
 // q = (bit t) + 2 (bit t+1).
