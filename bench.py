@@ -782,10 +782,10 @@ def run_paper_workload(args, rank, world, local):
             "gpu_launches": sum(v["launches"] for v in prof.values()),
             "time_share": {c_: round(v["ms"] / total, 4) for c_, v in prof.items() if v["launches"]},
             "clocks": clk}
-    if p["launches"]:  # the pass kernel against the measured HBM copy bandwidth (16 B per entry per pass)
+    if p["launches"]:  # the pass kernel against the measured HBM copy bandwidth (16 B per visited entry per pass)
         pk = os.path.join(ROOT, "MEASURED_PEAKS.json")
         hbm_peak = (json.load(open(pk)).get("hbm_gbs") if os.path.exists(pk) else None) or 6800.0
-        ach = 16.0 * 2.0 ** 35 / (p["ms"] / p["launches"] / 1e3) / 1e9
+        ach = p["bytes"] / (p["ms"] / 1e3) / 1e9
         line["roofline"] = {"bound": "hbm", "kernel": "pass_kernel", "achieved": ach, "peak": hbm_peak,
                             "unit": "GB/s", "frac": ach / hbm_peak, "pass_launches": p["launches"]}
     if rank == 0:

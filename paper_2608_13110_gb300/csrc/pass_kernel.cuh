@@ -396,7 +396,7 @@ __host__ __device__ constexpr int step_kind(int i) {
 // alone, cycles per tile: 9-bit forward window 6030 -> 5620, reversed 6510 -> 6100,
 // 7-bit top turn 7900 -> 7320, 9-bit top turn 11150 -> 10360, 8-bit window forward
 // 5300 -> 4860, 10-bit bottom turn 13150 -> 13120 (its lane steps and block
-// dominate). n=28, d=42, dense gates, 32 bitstrings: 6.00 -> 5.78 ms; n=70, d=56,
+// dominate). n=28, d=42, dense gates, 16 bitstrings: 6.00 -> 5.78 ms; n=70, d=56,
 // two bitstrings: 131.8 -> 128.2 ms.
 // Not the first step, which carries the rescale; small tiles have one tile per
 // CTA, where the time is set-up and latency (367 and 361 us on n=33, d=35, no
