@@ -536,30 +536,68 @@ int run_device(const Plan& P, const uint8_t* d_bits, int64_t nb, void* d_ws, int
     return TB_OK;
 }
 
-// Pinned staging of the synchronous entry, one block per host thread, allocated
-// at the thread's first call and freed with the thread: every call ends with a
-// stream synchronisation, so a block is never in use by two calls. Small calls
-// make one copy in each direction through it; pageable copies of the tables, the
-// bitstrings, the amplitudes and the fault word took most of a short call
-// (n=12, d=8, 64 bitstrings: 56 -> 43 us; n=33, d=35, one: 416 -> 402 us).
+// Pinned staging of the synchronous entry: blocks that the process keeps and calls
+// borrow. Every call ends with a stream synchronisation, so a block given back is
+// in nobody's use. Small calls make one copy in each direction through it;
+// pageable copies of the tables, the bitstrings, the amplitudes and the fault word
+// took most of a short call (n=12, d=8, 64 bitstrings: 56 -> 43 us; n=33, d=35,
+// one: 416 -> 402 us). The blocks belong to no thread: freeing pinned memory waits
+// for the whole device, so a thread that took its block along when it ended waited
+// for every other stream's work (a 0.1 ms call: 106 ms beside a stream with that much work, 0.13 ms now).
+// Calls that find no block copy from and to pageable memory.
 constexpr int64_t PINNED_BYTES = (int64_t)256 << 10;
-struct Pinned {
-    uint8_t* p = nullptr;
-    bool tried = false;
-    uint8_t* get() {
-        if (!tried) {
-            tried = true;
-            void* q = nullptr;
-            if (cudaHostAlloc(&q, (size_t)PINNED_BYTES, cudaHostAllocPortable) == cudaSuccess) p = static_cast<uint8_t*>(q);
-            else (void)cudaGetLastError();  // no pinned memory: the calls copy from and to pageable memory
+constexpr int PINNED_BLOCKS = 16;  // 4 MiB at most
+class PinnedPool {
+public:
+    uint8_t* take() {
+        {
+            std::lock_guard<std::mutex> lk(mu_);
+            if (nfree_ > 0) return free_[--nfree_];
+            if (closed_ || made_ == PINNED_BLOCKS) return nullptr;
+            ++made_;  // counted also when the allocation fails: a bounded number of attempts
         }
-        return p;
+        void* q = nullptr;
+        if (cudaHostAlloc(&q, (size_t)PINNED_BYTES, cudaHostAllocPortable) == cudaSuccess) return static_cast<uint8_t*>(q);
+        (void)cudaGetLastError();
+        return nullptr;
     }
-    ~Pinned() {
-        if (p) cudaFreeHost(p);
+    void give(uint8_t* p) {
+        std::lock_guard<std::mutex> lk(mu_);
+        free_[nfree_++] = p;
+    }
+    // The library is unloaded: free what no call holds.
+    void close() {
+        std::lock_guard<std::mutex> lk(mu_);
+        closed_ = true;
+        while (nfree_ > 0) (void)cudaFreeHost(free_[--nfree_]);
+    }
+
+private:
+    std::mutex mu_;
+    uint8_t* free_[PINNED_BLOCKS] = {};
+    int nfree_ = 0, made_ = 0;
+    bool closed_ = false;
+};
+PinnedPool g_pinned;  // no destructor of its own: a call on another thread may outlast the closer
+struct PinnedCloser {
+    ~PinnedCloser() { g_pinned.close(); }
+} g_pinned_closer;
+
+// A borrowed block (p, null: none). A call that fails half-way leaves no copy of
+// it in flight.
+struct PinnedLease {
+    uint8_t* p;
+    cudaStream_t st;
+    bool in_flight = true;
+    PinnedLease(bool wanted, cudaStream_t s) : p(wanted ? g_pinned.take() : nullptr), st(s) {}
+    PinnedLease(const PinnedLease&) = delete;
+    PinnedLease& operator=(const PinnedLease&) = delete;
+    ~PinnedLease() {
+        if (!p) return;
+        if (in_flight) (void)cudaStreamSynchronize(st);
+        g_pinned.give(p);
     }
 };
-thread_local Pinned t_pinned;
 
 }  // namespace rt
 }  // namespace tb
@@ -740,14 +778,8 @@ int tb_amplitudes(const tb_plan* plan, const uint8_t* bits, int64_t nb, void* d_
     // staged in the workspace: tables | bitstrings | amplitudes | fault word
     const int64_t in_bytes = nb * in_row(P), out_bytes = 16 * nb * amps_per_row(P);
     const int64_t out_off = P.lay.total + align_up(in_bytes, 256), back_bytes = align_up(out_bytes, 256) + sizeof(int);
-    uint8_t* pin = std::min(P.lay.total + stage, back_bytes) <= PINNED_BYTES ? t_pinned.get() : nullptr;
-    struct Settle {  // a call that fails half-way leaves no copy of the staging block in flight
-        cudaStream_t st;
-        bool on;
-        ~Settle() {
-            if (on) (void)cudaStreamSynchronize(st);
-        }
-    } settle{st, pin != nullptr};
+    PinnedLease lease(std::min(P.lay.total + stage, back_bytes) <= PINNED_BYTES, st);
+    uint8_t* const pin = lease.p;
     if (pin && P.lay.total + stage <= PINNED_BYTES) {
         std::memcpy(pin, P.blob.data(), (size_t)P.lay.total);
         std::memcpy(pin + P.lay.total, bits, (size_t)in_bytes);
@@ -764,14 +796,14 @@ int tb_amplitudes(const tb_plan* plan, const uint8_t* bits, int64_t nb, void* d_
     if (pin && back_bytes <= PINNED_BYTES) {  // amplitudes and fault word are neighbours
         TB_CUDA(cudaMemcpyAsync(pin, ws + out_off, (size_t)back_bytes, cudaMemcpyDeviceToHost, st));
         TB_CUDA(cudaStreamSynchronize(st));
-        settle.on = false;
+        lease.in_flight = false;
         std::memcpy(out, pin, (size_t)out_bytes);
         faults = *reinterpret_cast<const int*>(pin + back_bytes - sizeof(int));
     } else {
         TB_CUDA(cudaMemcpyAsync(out, d_out, (size_t)out_bytes, cudaMemcpyDeviceToHost, st));
         TB_CUDA(cudaMemcpyAsync(&faults, d_fault, sizeof(int), cudaMemcpyDeviceToHost, st));
         TB_CUDA(cudaStreamSynchronize(st));
-        settle.on = false;
+        lease.in_flight = false;
     }
     faults = note_faults(faults);
     t_last_faults = faults;
