@@ -7,6 +7,7 @@
 // are evaluated side by side when the workspace holds several boundaries.
 #include <cmath>
 #include <cstdio>
+#include <cstdlib>
 #include <cstring>
 #include <mutex>
 #include <new>
@@ -544,7 +545,10 @@ int run_device(const Plan& P, const uint8_t* d_bits, int64_t nb, void* d_ws, int
 // one: 416 -> 402 us). The blocks belong to no thread: freeing pinned memory waits
 // for the whole device, so a thread that took its block along when it ended waited
 // for every other stream's work (a 0.1 ms call: 106 ms beside a stream with that much work, 0.13 ms now).
-// Calls that find no block copy from and to pageable memory.
+// Calls that find no block copy from and to pageable memory. A block is host memory
+// of its own, registered with the driver: cudaDeviceReset unmaps what cudaHostAlloc
+// gave out, after which the next call would write to unmapped memory; a registered
+// block is pageable from then on and stays correct.
 constexpr int64_t PINNED_BYTES = (int64_t)256 << 10;
 constexpr int PINNED_BLOCKS = 16;  // 4 MiB at most
 class PinnedPool {
@@ -556,9 +560,11 @@ public:
             if (closed_ || made_ == PINNED_BLOCKS) return nullptr;
             ++made_;  // counted also when the allocation fails: a bounded number of attempts
         }
-        void* q = nullptr;
-        if (cudaHostAlloc(&q, (size_t)PINNED_BYTES, cudaHostAllocPortable) == cudaSuccess) return static_cast<uint8_t*>(q);
+        void* q = std::aligned_alloc(4096, (size_t)PINNED_BYTES);
+        if (q && cudaHostRegister(q, (size_t)PINNED_BYTES, cudaHostRegisterPortable) == cudaSuccess)
+            return static_cast<uint8_t*>(q);
         (void)cudaGetLastError();
+        std::free(q);
         return nullptr;
     }
     void give(uint8_t* p) {
@@ -569,7 +575,10 @@ public:
     void close() {
         std::lock_guard<std::mutex> lk(mu_);
         closed_ = true;
-        while (nfree_ > 0) (void)cudaFreeHost(free_[--nfree_]);
+        while (nfree_ > 0) {
+            (void)cudaHostUnregister(free_[--nfree_]);
+            std::free(free_[nfree_]);
+        }
     }
 
 private:
