@@ -271,6 +271,7 @@ int run_device(const Plan& P, const uint8_t* d_bits, int64_t nb, void* d_ws, int
         sp.n = P.n;
         sp.h = P.h;
         sp.nsm = num_sms();
+        sp.wide = P.wide_range ? 1 : 0;
         sp.bits = d_bits;
         sp.steps = tab<StepG>(d_ws, L.steps);
         sp.xq = tab<int16_t>(d_ws, L.step_xq);

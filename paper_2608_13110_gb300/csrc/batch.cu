@@ -118,6 +118,7 @@ int tb_batch_create(const tb_batch_item* items, int nitems, void* d_ws, int64_t 
         si.p.n = P.n;
         si.p.h = P.h;
         si.p.nb = (int)items[i].nb;
+        si.p.wide = P.wide_range ? 1 : 0;
         si.p.bits = items[i].d_bits;
         si.p.steps = at<StepG>(base, T.steps);
         si.p.xq = at<int16_t>(base, T.step_xq);

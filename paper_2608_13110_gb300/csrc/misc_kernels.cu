@@ -250,13 +250,19 @@ cudaError_t launch_finalize(const FinalizeParams& p, cudaStream_t st) {
 // 49 / 49 / 109, width 10 240 / 279 / 1234 -> 62 / 82 / 434, width 11
 // 365 / 456 / 2353 -> 101 / 135 / 807, width 12 604 / 817 / 4771 -> 144 / 237 / 1770.
 // Power-of-two rescaling (exact) at every turn, folded into the next window's
-// first coefficients.
+// first coefficients. Two things about that want gates near a unit scale: a
+// coefficient times the scale may leave FP32's range although its products do not
+// (growth by 2^80, then a gate of 2^-80), and a turn window runs two rows' steps
+// without a rescale. WIDE, for plans with other gates (Plan::wide_range), scales the
+// entries as the next window loads them and rescales between the rows of a turn
+// window too. A form of its own: scaling entries alone cost the ordinary plans 10 %
+// at width 8 and 8 % at width 10 with one bitstring.
 template <int H, int RW>
 struct Narrow {
     static constexpr int T = 1 << (H - RW - 1);  // threads
     static constexpr int NK = 1 << RW;           // packed pairs per thread
-    static constexpr int MID = H - 2 * RW;       // bits between the two turn windows
     static constexpr int NW = (T + 31) / 32;
+    static_assert(H > 2 * RW, "a window between the two turn windows takes the rescale");
     // spectator bit of the window [lo, lo + RW): neither in it nor next to it,
     // and not among the lowest bits, which the lanes hold
     static constexpr int vbit(int lo) { return lo + RW + 1 <= H - 1 ? H - 1 : lo - 2; }
@@ -349,7 +355,7 @@ __device__ __forceinline__ void narrow_rev(float2 (&P)[NK], float2 (&Q)[NK], con
     }
 }
 
-template <int H, int RW>
+template <int H, int RW, bool WIDE>
 struct NarrowRun {
     using W = Narrow<H, RW>;
     static constexpr int NK = W::NK, T = W::T;
@@ -436,14 +442,30 @@ struct NarrowRun {
         S += s;
         return ldexpf(1.0f, s);
     }
-    // targets of the middle windows, RW at a time; the first one is rescaled
+    __device__ __forceinline__ static void scale_by(float2 (&P)[NK], float2 (&Q)[NK], float s) {
+#pragma unroll
+        for (int k = 0; k < NK; ++k) {
+            P[k] = __fmul2_rn(P[k], make_float2(s, s));
+            Q[k] = __fmul2_rn(Q[k], make_float2(s, s));
+        }
+    }
+    // WIDE: rescale in registers, between the two rows of a turn window
+    __device__ __forceinline__ void rescale_row(float2 (&P)[NK], float2 (&Q)[NK], int& turn) {
+        if constexpr (WIDE) {
+            put_max(reg_max(P, Q), ++turn);
+            sync();
+            scale_by(P, Q, take_scale(turn));
+        }
+    }
+    // targets of the middle windows, RW at a time; SC: the first one is rescaled
     template <bool SC, int T0>
     __device__ __forceinline__ void mid_fwd(const float2* c, float s) {
         if constexpr (T0 < H - RW) {
             constexpr int N = (H - RW - T0) < RW ? (H - RW - T0) : RW;
             float2 P[NK], Q[NK];
             load<T0>(P, Q);
-            narrow_fwd<SC, NK, T0, T0, N>(P, Q, c, addr<T0>(), s);
+            if constexpr (SC && WIDE) scale_by(P, Q, s);
+            narrow_fwd<SC && !WIDE, NK, T0, T0, N>(P, Q, c, addr<T0>(), s);
             store<T0>(P, Q);
             sync();
             mid_fwd<false, T0 + N>(c, 1.0f);
@@ -456,7 +478,8 @@ struct NarrowRun {
             constexpr int LO = T0 - RW + 1;
             float2 P[NK], Q[NK];
             load<LO>(P, Q);
-            narrow_rev<SC, NK, RW, H, LO, T0, N>(P, Q, c, addr<LO>(), s);
+            if constexpr (SC && WIDE) scale_by(P, Q, s);
+            narrow_rev<SC && !WIDE, NK, RW, H, LO, T0, N>(P, Q, c, addr<LO>(), s);
             store<LO>(P, Q);
             sync();
             mid_rev<false, T0 - N>(c, 1.0f);
@@ -481,11 +504,7 @@ struct NarrowRun {
         if (p.nrows > 0) {
             float2 P[NK], Q[NK];
             load<0>(P, Q);
-#pragma unroll
-            for (int k = 0; k < NK; ++k) {
-                P[k] = __fmul2_rn(P[k], make_float2(s, s));
-                Q[k] = __fmul2_rn(Q[k], make_float2(s, s));
-            }
+            scale_by(P, Q, s);
             for (int cyc = 0;; ++cyc) {
                 const float2* c = cf + (cyc & 1) * 2 * ROW_CF;
                 fetch(cyc + 1);
@@ -494,28 +513,30 @@ struct NarrowRun {
                 store<0>(P, Q);
                 sync();
                 s = take_scale(turn);
-                if constexpr (W::MID > 0) mid_fwd<true, RW>(c, s);
+                mid_fwd<true, RW>(c, s);
                 load<TOP>(P, Q);
-                narrow_fwd<W::MID == 0, NK, TOP, TOP, RW>(P, Q, c, addr<TOP>(), s);
+                narrow_fwd<false, NK, TOP, TOP, RW>(P, Q, c, addr<TOP>(), 1.0f);
                 if (++row == p.nrows) {
                     put_max(reg_max(P, Q), ++turn);
                     store<TOP>(P, Q);
                     break;
                 }
+                rescale_row(P, Q, turn);
                 narrow_rev<false, NK, RW, H, TOP, H - 1, RW>(P, Q, c + ROW_CF, 0u, 1.0f);
                 put_max(reg_max(P, Q), ++turn);
                 store<TOP>(P, Q);
                 stage(cyc + 1);
                 sync();
                 s = take_scale(turn);
-                if constexpr (W::MID > 0) mid_rev<true, H - RW - 1>(c + ROW_CF, s);
+                mid_rev<true, H - RW - 1>(c + ROW_CF, s);
                 load<0>(P, Q);
-                narrow_rev<W::MID == 0, NK, RW, H, 0, RW - 1, RW>(P, Q, c + ROW_CF, addr<0>(), s);
+                narrow_rev<false, NK, RW, H, 0, RW - 1, RW>(P, Q, c + ROW_CF, addr<0>(), 1.0f);
                 if (++row == p.nrows) {
                     put_max(reg_max(P, Q), ++turn);
                     store<0>(P, Q);
                     break;
                 }
+                rescale_row(P, Q, turn);
             }
             sync();
             s = take_scale(turn);
@@ -700,12 +721,12 @@ constexpr int narrow_smem(int h, bool few) {  // boundary, coefficients, reducti
     return h < 8 ? 0 : (8 << h) + 2 * 2 * h * NARROW_CF * 8 + (narrow_threads(h, few) / 32) * 24;
 }
 
-template <int H, bool FEW>
+template <int H, bool FEW, bool WIDE>
 __device__ __forceinline__ void narrow_sweep(const SmallParams& p, int b, uint8_t* smem) {
     if constexpr (H < 8) {
         if (threadIdx.x < 32) narrow_warp<H>(p, b);
     } else {
-        using R = NarrowRun<H, narrow_rw(H, FEW)>;
+        using R = NarrowRun<H, narrow_rw(H, FEW), WIDE>;
         static_assert(R::T >= 32, "whole warps");
         if (threadIdx.x >= R::T) return;
         float2* Bs = reinterpret_cast<float2*>(smem);
@@ -716,10 +737,10 @@ __device__ __forceinline__ void narrow_sweep(const SmallParams& p, int b, uint8_
     }
 }
 
-template <int H, bool FEW>
+template <int H, bool FEW, bool WIDE>
 __global__ void __launch_bounds__(narrow_threads(H, FEW)) narrow_kernel(const __grid_constant__ SmallParams p) {
     extern __shared__ __align__(16) uint8_t nsm[];
-    narrow_sweep<H, FEW>(p, blockIdx.x, nsm);
+    narrow_sweep<H, FEW, WIDE>(p, blockIdx.x, nsm);
 }
 
 // Several narrow plans in one launch: block i evaluates bitstring
@@ -739,18 +760,18 @@ __global__ void __launch_bounds__(NARROW_MULTI_THREADS) narrow_multi_kernel(cons
     const SmallParams p = items[lo].p;
     const int b = (int)(blk - items[lo].first_block);
     switch (p.h) {
-        case 1: narrow_sweep<1, false>(p, b, nsm); break;
-        case 2: narrow_sweep<2, false>(p, b, nsm); break;
-        case 3: narrow_sweep<3, false>(p, b, nsm); break;
-        case 4: narrow_sweep<4, false>(p, b, nsm); break;
-        case 5: narrow_sweep<5, false>(p, b, nsm); break;
-        case 6: narrow_sweep<6, false>(p, b, nsm); break;
-        case 7: narrow_sweep<7, false>(p, b, nsm); break;
-        case 8: narrow_sweep<8, false>(p, b, nsm); break;
-        case 9: narrow_sweep<9, false>(p, b, nsm); break;
-        case 10: narrow_sweep<10, false>(p, b, nsm); break;
-        case 11: narrow_sweep<11, false>(p, b, nsm); break;
-        case 12: narrow_sweep<12, false>(p, b, nsm); break;
+        case 1: narrow_sweep<1, false, false>(p, b, nsm); break;
+        case 2: narrow_sweep<2, false, false>(p, b, nsm); break;
+        case 3: narrow_sweep<3, false, false>(p, b, nsm); break;
+        case 4: narrow_sweep<4, false, false>(p, b, nsm); break;
+        case 5: narrow_sweep<5, false, false>(p, b, nsm); break;
+        case 6: narrow_sweep<6, false, false>(p, b, nsm); break;
+        case 7: narrow_sweep<7, false, false>(p, b, nsm); break;
+        case 8: p.wide ? narrow_sweep<8, false, true>(p, b, nsm) : narrow_sweep<8, false, false>(p, b, nsm); break;
+        case 9: p.wide ? narrow_sweep<9, false, true>(p, b, nsm) : narrow_sweep<9, false, false>(p, b, nsm); break;
+        case 10: p.wide ? narrow_sweep<10, false, true>(p, b, nsm) : narrow_sweep<10, false, false>(p, b, nsm); break;
+        case 11: p.wide ? narrow_sweep<11, false, true>(p, b, nsm) : narrow_sweep<11, false, false>(p, b, nsm); break;
+        case 12: p.wide ? narrow_sweep<12, false, true>(p, b, nsm) : narrow_sweep<12, false, false>(p, b, nsm); break;
         default: break;
     }
 }
@@ -762,11 +783,19 @@ cudaError_t launch_small_multi(const SmallItem* d_items, int nitems, int64_t nbl
     return cudaGetLastError();
 }
 
+template <int H, bool WIDE>
+cudaError_t launch_form(const SmallParams& p, cudaStream_t st) {
+    if (p.nb <= p.nsm) narrow_kernel<H, true, WIDE><<<p.nb, narrow_threads(H, true), narrow_smem(H, true), st>>>(p);
+    else narrow_kernel<H, false, WIDE><<<p.nb, narrow_threads(H, false), narrow_smem(H, false), st>>>(p);
+    return cudaGetLastError();
+}
+
 template <int H>
 cudaError_t launch_narrow(const SmallParams& p, cudaStream_t st) {
-    if (p.nb <= p.nsm) narrow_kernel<H, true><<<p.nb, narrow_threads(H, true), narrow_smem(H, true), st>>>(p);
-    else narrow_kernel<H, false><<<p.nb, narrow_threads(H, false), narrow_smem(H, false), st>>>(p);
-    return cudaGetLastError();
+    if constexpr (H >= 8) {  // narrower boundaries rescale after every row as they are
+        if (p.wide) return launch_form<H, true>(p, st);
+    }
+    return launch_form<H, false>(p, st);
 }
 
 cudaError_t launch_small(const SmallParams& p, cudaStream_t st) {

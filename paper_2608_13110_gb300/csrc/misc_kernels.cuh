@@ -54,6 +54,7 @@ struct FinalizeParams {
 struct SmallParams {
     int n, h, nb;
     int nsm;               // SMs of the device
+    int wide;              // Plan::wide_range
     const uint8_t* bits;
     const StepG* steps;
     const int16_t* xq;

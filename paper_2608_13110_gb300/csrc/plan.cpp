@@ -624,6 +624,16 @@ int plan_build(Plan& P, int n, int d, const uint8_t* cliff, const uint8_t* tmask
         u = m2_mul(E, u);
     }
     auto U = [&](int q, int t) -> const M2& { return P.U[(size_t)t * n + q]; };
+    // Gates far from a unit scale: a singular value outside [1/2, 2]. Within it a
+    // step of the sweep grows the boundary by 2^5 at most, 16 steps in a row by 2^80.
+    P.wide_range = false;
+    for (const M2& u : P.U) {
+        double f = 0.0;  // sum and product of the squared singular values
+        for (const cd& z : u.a) f += std::norm(z);
+        const double det2 = std::norm(u.a[0] * u.a[3] - u.a[1] * u.a[2]);
+        const double root = std::sqrt(std::max(0.0, f * f - 4.0 * det2));
+        if (!(f + root <= 8.0 && f - root >= 0.5)) P.wide_range = true;
+    }
 
     // ---- entanglers: CZ, or diag(1, 1, 1, e^(i phi)) per gate (phi = pi is CZ exactly)
     P.W.assign((size_t)d * (n - 1), cd(-1.0, 0.0));

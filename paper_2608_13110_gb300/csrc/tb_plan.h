@@ -50,6 +50,7 @@ struct Plan {
     std::vector<float2> open_w;  // entangler factor w of each late crossing (-1 for CZ)
     TileSkip join_skip{};              // 128-row blocks the tensor-core join visits
     std::vector<LateSkip> late_skip;   // rows each late crossing writes and reads
+    bool wide_range = false;  // some one-qubit gate is far from unitary scale
     int last_mid_row() const { return open_k ? n - open_k - 1 : n - 2; }
     int n_pass_launches() const {
         return opts.precision != TB_PRECISION_FP32 ? (int)tc_passes.size() : (int)passes.size();
