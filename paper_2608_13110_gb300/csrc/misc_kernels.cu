@@ -235,6 +235,16 @@ cudaError_t launch_finalize(const FinalizeParams& p, cudaStream_t st) {
 // (and im alike), whatever the layout below.
 // ---------------------------------------------------------------------------
 
+// Window bits at width h. few: the bitstrings fit one CTA per SM, so the length
+// of one sweep counts (fewer entries per thread, more warps); otherwise the
+// FP32 pipe counts (more steps per window). Measured with 1 / 256 / 512
+// bitstrings at n = 45 (us, before the last refinements): width 11 with RW = 2
+// 109 / 180 / 349, 3 124 / 151 / 308; width 12 with RW = 3 164 / 322 / 634,
+// 4 195 / 259 / 538; at widths 8 to 10 RW = 2 is the best for both (width 10:
+// 70 / 91 / 154, RW = 3 117 / 122 / 167).
+constexpr int narrow_rw(int h, bool few) { return h <= 10 ? 2 : h == 11 ? (few ? 2 : 3) : (few ? 3 : 4); }
+constexpr int narrow_threads(int h, bool few) { return h < 8 ? 32 : 1 << (h - narrow_rw(h, few) - 1); }
+
 // --- 8 <= h <= 12: register windows ----------------------------------------
 // A thread holds 2^(RW+1) entries in registers: RW consecutive address bits
 // (the window) and one spectator bit v whose two values share a packed pair
@@ -362,6 +372,10 @@ struct NarrowRun {
     static constexpr int ROW_CF = H * NARROW_CF;       // a row's packed coefficients
     static constexpr int CYCLE = 2 * H * 8;            // raw coefficients of two rows
     static constexpr int PRE = (CYCLE + T - 1) / T;    // of which a thread stages this many
+    // The last row's FP64 sum: as many strided partial sums as the few-bitstring form
+    // has threads, added in the same order in every form, so that an amplitude does
+    // not depend on how many bitstrings share the call.
+    static constexpr int GROUPS = narrow_threads(H, true) / T;
     float2* Bs;
     float2* cf;     // [2 buffers][2 rows][H][NARROW_CF]
     float* red;     // [2][NW]
@@ -542,23 +556,32 @@ struct NarrowRun {
             s = take_scale(turn);
         }
         const int xl = xb[p.n - 1] ? 1 : 0;
-        double ar = 0.0, ai = 0.0;
-        for (int e = (int)t; e < N; e += T) {
-            const float2 z = Bs[W::swz((uint32_t)e)];
-            const float2 v = cmul(make_float2(z.x * s, z.y * s), p.red_low[2 * e + xl]);
-            ar += (double)v.x;
-            ai += (double)v.y;
+        double ar[GROUPS] = {}, ai[GROUPS] = {};
+        for (int e0 = (int)t; e0 < N; e0 += GROUPS * T) {
+#pragma unroll
+            for (int g = 0; g < GROUPS; ++g) {
+                const int e = e0 + g * T;
+                const float2 z = Bs[W::swz((uint32_t)e)];
+                const float2 v = cmul(make_float2(z.x * s, z.y * s), p.red_low[2 * e + xl]);
+                ar[g] += (double)v.x;
+                ai[g] += (double)v.y;
+            }
         }
 #pragma unroll
         for (int off = 16; off > 0; off >>= 1) {
-            ar += __shfl_xor_sync(0xffffffffu, ar, off);
-            ai += __shfl_xor_sync(0xffffffffu, ai, off);
+#pragma unroll
+            for (int g = 0; g < GROUPS; ++g) {
+                ar[g] += __shfl_xor_sync(0xffffffffu, ar[g], off);
+                ai[g] += __shfl_xor_sync(0xffffffffu, ai[g], off);
+            }
         }
-        if ((t & 31) == 0) redd[t >> 5] = make_double2(ar, ai);
+#pragma unroll
+        for (int g = 0; g < GROUPS; ++g)
+            if ((t & 31) == 0) redd[g * W::NW + (t >> 5)] = make_double2(ar[g], ai[g]);
         sync();
         if (t == 0) {
             double2 tot = redd[0];
-            for (int i = 1; i < W::NW; ++i) { tot.x += redd[i].x; tot.y += redd[i].y; }
+            for (int i = 1; i < GROUPS * W::NW; ++i) { tot.x += redd[i].x; tot.y += redd[i].y; }
             const int Si = (int)max(-1000000LL, min(1000000LL, S));
             p.out[2 * b] = scalbn(tot.x, -Si);
             p.out[2 * b + 1] = scalbn(tot.y, -Si);
@@ -708,17 +731,9 @@ __device__ void narrow_warp(const SmallParams& p, int b) {
     }
 }
 
-// Window bits at width h. few: the bitstrings fit one CTA per SM, so the length
-// of one sweep counts (fewer entries per thread, more warps); otherwise the
-// FP32 pipe counts (more steps per window). Measured with 1 / 256 / 512
-// bitstrings at n = 45 (us, before the last refinements): width 11 with RW = 2
-// 109 / 180 / 349, 3 124 / 151 / 308; width 12 with RW = 3 164 / 322 / 634,
-// 4 195 / 259 / 538; at widths 8 to 10 RW = 2 is the best for both (width 10:
-// 70 / 91 / 154, RW = 3 117 / 122 / 167).
-constexpr int narrow_rw(int h, bool few) { return h <= 10 ? 2 : h == 11 ? (few ? 2 : 3) : (few ? 3 : 4); }
-constexpr int narrow_threads(int h, bool few) { return h < 8 ? 32 : 1 << (h - narrow_rw(h, few) - 1); }
 constexpr int narrow_smem(int h, bool few) {  // boundary, coefficients, reduction scratch of every warp
-    return h < 8 ? 0 : (8 << h) + 2 * 2 * h * NARROW_CF * 8 + (narrow_threads(h, few) / 32) * 24;
+    return h < 8 ? 0 : (8 << h) + 2 * 2 * h * NARROW_CF * 8 + (narrow_threads(h, true) / 32) * 16 +
+                           (narrow_threads(h, few) / 32) * 8;
 }
 
 template <int H, bool FEW, bool WIDE>
@@ -731,8 +746,8 @@ __device__ __forceinline__ void narrow_sweep(const SmallParams& p, int b, uint8_
         if (threadIdx.x >= R::T) return;
         float2* Bs = reinterpret_cast<float2*>(smem);
         float2* cf = Bs + (1 << H);
-        double2* redd = reinterpret_cast<double2*>(cf + 2 * 2 * R::ROW_CF);  // [NW], then red [2][NW]
-        R r{Bs, cf, reinterpret_cast<float*>(redd + R::W::NW), p, p.bits + (int64_t)b * p.n, threadIdx.x, 0, {}};
+        double2* redd = reinterpret_cast<double2*>(cf + 2 * 2 * R::ROW_CF);  // [GROUPS][NW], then red [2][NW]
+        R r{Bs, cf, reinterpret_cast<float*>(redd + R::GROUPS * R::W::NW), p, p.bits + (int64_t)b * p.n, threadIdx.x, 0, {}};
         r.run(b, redd);
     }
 }
