@@ -431,13 +431,61 @@ private:
     int n_ = 0;
 };
 
+// Whether a zero entry stays zero whatever it is multiplied with: 0 x inf is not 0.
+// Every table that the device reads is finite in FP32 (gates of rows 0 and n-1 and of
+// the open band included), and no product of tables and no pass, which starts from
+// entries below 1, can leave FP32's range.
+static bool zeros_last(const Plan& P) {
+    constexpr double LIMIT = 1e37;
+    auto top = [](const void* v, size_t n) {  // largest magnitude of n floats; inf for inf and NaN
+        const uint8_t* b = static_cast<const uint8_t*>(v);
+        uint32_t m = 0;  // magnitudes compare like their bits
+        for (size_t i = 0; i < n; ++i) {
+            uint32_t u;
+            std::memcpy(&u, b + 4 * i, 4);
+            m = std::max(m, u & 0x7fffffffu);
+        }
+        float f;
+        std::memcpy(&f, &m, 4);
+        return m >= 0x7f800000u ? HUGE_VAL : (double)f;
+    };
+    auto tab = [&](const std::vector<float2>& t) { return top(t.data(), 2 * t.size()); };
+    auto steps = [&](const std::vector<StepG>& t) { return top(t.data(), 32 * t.size()); };
+    static_assert(sizeof(StepG) == 32 * sizeof(float), "StepG is read as floats");
+    // complex products: twice the real product of the magnitudes
+    if (!(tab(P.init_low) * std::max(1.0, 2.0 * tab(P.init_mid)) * std::max(1.0, 2.0 * tab(P.init_top)) <= LIMIT)) return false;
+    if (!(std::max(1.0, tab(P.red_mid)) * 4.0 * tab(P.red_top) <= LIMIT && tab(P.red_low) <= LIMIT)) return false;
+    if (!(steps(P.steps) <= LIMIT && steps(P.pass_steps) <= LIMIT && tab(P.open_E) <= LIMIT && tab(P.open_w) <= LIMIT))
+        return false;
+    for (const OpenOp& o : P.open_ops)
+        if (!(top(o.m, o.kind == 0 ? 8 : 2) <= LIMIT)) return false;  // a gate, or its factor
+    // split blocks: TF32 values are floats, BF16 values the upper halves of floats
+    if (P.opts.precision == TB_PRECISION_TF32X3) {
+        if (!(top(P.tc_mats.data(), P.tc_mats.size() / 4) <= LIMIT)) return false;
+    } else if (!P.tc_mats.empty()) {
+        const uint16_t* v = reinterpret_cast<const uint16_t*>(P.tc_mats.data());
+        bool bad = false;
+        for (size_t i = 0; i < P.tc_mats.size() / 2; ++i) bad |= (v[i] & 0x7f80u) >= 0x7e80u;  // 2^126 and above
+        if (bad) return false;
+    }
+    // growth within a pass: two products of complex values a step
+    auto grows = [&](int step0, int n) {
+        double g = 0.0;
+        for (int i = step0; i < std::min(step0 + n, (int)P.steps.size()); ++i)
+            g += std::max(0.0, std::log2(4.0 * top(P.steps[i].g, 32)));
+        return !(g <= 120.0);
+    };
+    for (size_t k = 0; k < P.passes.size(); ++k)
+        if (grows(P.passes[k].step0, P.passes[k].nsteps + (pass_blk(P.passes[k].type, P.passes[k].M) >= 0 ? 3 : 0))) return false;
+    for (const TcPass& d : P.tc_passes)
+        if (grows(d.step0, d.nsteps)) return false;
+    return true;
+}
+
 // Fill in every pass's TileSkip. row0: the support of the row-0 boundary.
 static void tile_skips(Plan& P, Support s) {
     const int h = P.h;
-    double z0 = 0.0;  // 0 x inf is not 0: non-finite gates leave every tile visited
-    for (const auto& g : P.steps64)
-        for (const cd& z : g) z0 += z.real() * 0.0 + z.imag() * 0.0;
-    const bool finite = z0 == 0.0;
+    const bool finite = zeros_last(P);
     if (!finite) s = Support();
     int done = 0;
     auto advance = [&](int end) {
