@@ -471,7 +471,7 @@ int run_device(const Plan& P, const uint8_t* d_bits, int64_t nb, void* d_ws, int
                 lp.out_stride = b_stride;
                 lp.in_shift = c.open_in_place ? i : 0;
                 lp.out_shift = c.open_in_place ? i + 1 : 0;
-                lp.out_entries = (int64_t)1 << (P.h - 1 - i);
+                lp.out_entries = P.late_rows((size_t)i) << k;
                 lp.nbatch = nbat;
                 lp.k = k;
                 lp.ops = ops + P.open_seg[i];

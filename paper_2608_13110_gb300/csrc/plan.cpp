@@ -528,8 +528,7 @@ static void tile_skips(Plan& P, Support s) {
         ls.mask = (uint32_t)(m >> (k + i + 1));
         ls.fix = (uint32_t)v;
         s.eliminate(k + (int)i);
-        // the last crossing's output is read in full (2^k entries, or twice
-        // that with an idle top bit)
+        // the last crossing writes the output, row 0 (Plan::late_rows)
         ls.out = i + 2 < P.open_seg.size() ? s.skip(h, k + (int)i + 1, -1, 0)
                                            : Support().skip(h, k + (int)i + 1, -1, 0);
         P.late_skip.push_back(ls);

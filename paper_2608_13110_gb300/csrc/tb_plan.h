@@ -50,6 +50,12 @@ struct Plan {
     std::vector<float2> open_w;  // entangler factor w of each late crossing (-1 for CZ)
     TileSkip join_skip{};              // 128-row blocks the tensor-core join visits
     std::vector<LateSkip> late_skip;   // rows each late crossing writes and reads
+    // Output rows (2^k entries) of late crossing i: half its input's. The last one
+    // writes row 0 alone, the output; an idle top bit (odd d and odd crossing layers)
+    // would make it two rows, the second from input rows that nothing writes.
+    int64_t late_rows(size_t i) const {
+        return i + 2 < open_seg.size() ? (int64_t)1 << (h - open_k - 1 - (int)i) : 1;
+    }
     bool wide_range = false;  // some one-qubit gate is far from unitary scale
     int last_mid_row() const { return open_k ? n - open_k - 1 : n - 2; }
     int n_pass_launches() const {
