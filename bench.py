@@ -351,7 +351,7 @@ def run_ours(args, rank, world, local):
                      "peak_source": f"{peak_src} copy bandwidth",
                      "pass_launches": p["launches"], "pass_ms_total": p["ms"],
                      "pass_share_of_kernel_time": p["ms"] / max(1e-9, sum(v["ms"] for v in prof.values())),
-                     "fma_pipe": fma_pipe_fraction(args, info, nb, h, p, clk, dev)},
+                     "fma_pipe": fma_pipe_fraction(args, plan, nb, p, clk, dev)},
         "clocks": clk,
         "sanity": {"log_xeb": tb.log_xeb(amps, c.n), "e2e_matches_device": bool(np.array_equal(amps, e2e_amps))},
     }
@@ -362,20 +362,19 @@ def run_ours(args, rank, world, local):
         print(json.dumps(line))
 
 
-def fma_pipe_fraction(args, info, nb, h, p, clk, dev):
+def fma_pipe_fraction(args, plan, nb, p, clk, dev):
     """The FP32 passes' other ceiling: the multiply-adds the pass kernels
-    spend per entry (8 per paired step, 16 per row turn's 4x4 block: the mean
-    of the plan's pass_madds over its passes), for the entries they visit, over
-    the pass kernels' measured time, against SMs x 128 FP32 lanes x the SM clock
-    (one FMA per lane and cycle; the paired FFMA2 issues two lanes' worth in two
-    cycles). Secondary to the HBM roofline: the two floors are within 15 % of
-    each other at width 32."""
+    execute (8 per entry and paired step, 16 per row turn's 4x4 block, without
+    the entries and warps left out as zero: the plan's own count), over their
+    measured time, against SMs x 128 FP32 lanes x the SM clock (one FMA per lane
+    and cycle; the paired FFMA2 issues two lanes' worth in two cycles).
+    Secondary to the HBM roofline."""
     if args.precision != "fp32" or p["ms"] <= 0:
         return None
     import torch
     sms = torch.cuda.get_device_properties(dev).multi_processor_count
     mhz = clk.get("sm_max_mhz") or 2070.0
-    fma = p["bytes"] / 16.0 * info["pass_madds"] / max(1, info["n_passes"])
+    fma = plan.visited[1] * nb * args.steps
     achieved = fma / (p["ms"] / 1e3) / 1e12
     peak = sms * 128 * mhz * 1e6 / 1e12
     return {"achieved": achieved, "peak": peak, "unit": "TFMA/s", "frac": achieved / peak,

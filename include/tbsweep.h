@@ -259,6 +259,15 @@ TB_API int tb_amplitudes(const tb_plan* plan, const uint8_t* bits, int64_t nb, v
  * or -1 for a NULL plan. */
 TB_API int tb_plan_schedule(const tb_plan* plan, int32_t* sched, int cap);
 
+/* What the passes of one amplitude really do once the entries known to be
+ * exactly zero are left out: *entries, the boundary entries that they read and
+ * write (16 bytes each; n_passes * 2^h when nothing is zero), and *madds, the
+ * real multiply-adds that the FP32 pass kernels execute on them (pass_madds *
+ * 2^h when nothing is zero; 0 for split-precision plans). A call on so few
+ * bitstrings that its passes run on small tiles also executes those of the
+ * zero warps, which madds leaves out. Either pointer may be NULL. */
+TB_API int tb_plan_visited(const tb_plan* plan, double* entries, double* madds);
+
 /* ---- Batches of circuits -------------------------------------------------
  * Many independent circuits (the paper evaluates many contractions of one
  * topology as independent jobs, Sec. 5.2; here n and d may differ) recorded

@@ -57,6 +57,7 @@ _sig = {
     "tb_amplitudes": (ctypes.c_int, [_vp, _u8p, ctypes.c_int64, _vp, ctypes.c_int64, _dp, _vp]),
     "tb_amplitudes_noalloc": (ctypes.c_int, [_vp, _vp, ctypes.c_int64, _vp, _vp]),
     "tb_plan_schedule": (ctypes.c_int, [_vp, ctypes.POINTER(ctypes.c_int32), ctypes.c_int]),
+    "tb_plan_visited": (ctypes.c_int, [_vp, _dp, _dp]),
     "tb_batch_workspace_bytes": (ctypes.c_int64, [ctypes.c_void_p, ctypes.c_int]),
     "tb_batch_create": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_int, _vp, ctypes.c_int64, ctypes.c_int, _vp,
                                        ctypes.POINTER(_vp)]),
@@ -289,6 +290,14 @@ class Plan:
         buf = (ctypes.c_int32 * max(1, 3 * npass))()
         _lib.tb_plan_schedule(self._h, buf, npass)
         return [(self.PASS_SHAPES[buf[3 * i]], buf[3 * i + 1], buf[3 * i + 2]) for i in range(npass)]
+
+    @property
+    def visited(self) -> tuple:
+        """(entries, multiply-adds): what the passes of one amplitude move and
+        execute once the entries known to be zero are left out."""
+        e, m = ctypes.c_double(), ctypes.c_double()
+        _check(_lib.tb_plan_visited(self._h, ctypes.byref(e), ctypes.byref(m)), "tb_plan_visited")
+        return e.value, m.value
 
     def workspace_bytes(self, nb: int) -> int:
         v = _lib.tb_workspace_bytes(self._h, int(nb))

@@ -732,6 +732,15 @@ int tb_plan_schedule(const tb_plan* plan, int32_t* sched, int cap) {
     return np;
 }
 
+int tb_plan_visited(const tb_plan* plan, double* entries, double* madds) {
+    if (!plan) return fail(TB_EINVAL, "NULL argument");
+    double e = 0.0, m = 0.0;
+    plan_visited(plan->p, &e, &m);
+    if (entries) *entries = e;
+    if (madds) *madds = m;
+    return TB_OK;
+}
+
 int64_t tb_workspace_bytes(const tb_plan* plan, int64_t nb) {
     if (!plan || nb < 0) return -1;
     const Plan& P = plan->p;

@@ -535,6 +535,17 @@ static void tile_skips(Plan& P, Support s) {
     }
 }
 
+void plan_visited(const Plan& P, double* entries, double* madds) {
+    *entries = *madds = 0.0;
+    for (const PassDesc& d : P.passes) {
+        const double e = std::ldexp(1.0, P.h - d.skip.n);
+        *entries += e;
+        // every equation of a WarpSkip idles half of the warps
+        *madds += std::ldexp(e, -d.warps.n) * (8 * d.nsteps + (pass_blk(d.type, d.M) >= 0 ? 8 : 0));
+    }
+    for (const TcPass& d : P.tc_passes) *entries += std::ldexp(1.0, P.h - d.skip.n);
+}
+
 // Modelled time of a schedule in units of one HBM pass, a heuristic for the
 // planner's default (the autotuner times candidates on the device): a pass
 // costs the larger of its memory time and its arithmetic time (alpha per

@@ -73,6 +73,9 @@ struct Plan {
     std::vector<uint8_t> blob;
 };
 
+// Entries that the passes of one amplitude move and multiply-adds that they execute.
+void plan_visited(const Plan& P, double* entries, double* madds);
+
 uint64_t next_plan_uid();
 
 // Early-region matrix and late-region operations of an open plan (open_plan.cpp).
