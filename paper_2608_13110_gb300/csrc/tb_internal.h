@@ -307,15 +307,6 @@ struct TableLayout {
     int64_t total;
 };
 
-// Per-bitstring rescaling state: slot 0 is written by the row-0 writer, slot
-// k+1 by pass k, slot P+1 by the last-row reduction.
-//   maxs[slot]: float bits of max(|re|, |im|) over the boundary after it
-//   exps[slot]: the power of two the producer multiplied its input by
-struct ScaleLayout {
-    int nslots;
-    int64_t bytes_per_b;  // maxs (uint32) then exps (int32), padded
-};
-
 #ifdef __CUDACC__
 // The kernels of one sweep follow one another on a stream and each needs all of
 // its predecessor's boundary, but not to set itself up: a kernel launched with

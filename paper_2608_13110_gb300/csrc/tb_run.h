@@ -23,9 +23,13 @@ int fail(int code, const std::string& msg);
 constexpr int64_t DEFAULT_BATCH_ENTRIES = (int64_t)1 << 30;  // 8 GiB of boundaries
 
 // Per-bitstring device bytes of the HBM-pass path (zero for narrow plans).
+// Rescaling state: slot 0 is written by the row-0 writer, slot k+1 by pass k, slot
+// P+1 by the last-row reduction.
+//   maxs[slot]: float bits of max(|re|, |im|) over the boundary after it
+//   exps[slot]: the power of two the producer multiplied its input by
 struct CallLayout {
     int nslots = 0;
-    int64_t scale_bytes = 0;     // rescaling slots
+    int64_t scale_bytes = 0;     // maxs (uint32) then exps (int32), padded
     int red_blocks = 0;          // reduction blocks
     int64_t partial_bytes = 0;   // reduction partial sums
     int64_t boundary_bytes = 0;  // the boundary, 8 * 2^h
