@@ -187,9 +187,14 @@ def kernel_code_hash() -> str:
     return hashlib.sha256(src.encode()).hexdigest()[:16]
 
 
+L2_BYTES = 129e6
+
+
 def pass_traffic(entries: float):
     """DRAM bytes per pass launch from the committed ncu summary, scaled to the
-    entries a pass visits, or None if absent or taken on other kernel sources."""
+    entries a pass visits, or None if absent, taken on other kernel sources, or
+    where either visited set is not far larger than the L2: what a smaller one
+    leaves there for the next pass says nothing about another size."""
     path = os.path.join(ROOT, "profiles", "pass_kernel_traffic.txt")
     if not os.path.exists(path):
         return None
@@ -202,6 +207,8 @@ def pass_traffic(entries: float):
     if kv.get("pass_kernel_code_sha256_16") != digest:
         return None
     try:
+        if min(float(kv["visited_bytes"]), 8.0 * entries) < 8.0 * L2_BYTES:
+            return None
         return float(kv["dram_bytes_per_entry"]) * entries
     except (KeyError, ValueError):
         return None
