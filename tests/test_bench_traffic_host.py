@@ -33,8 +33,3 @@ def test_a_summary_without_its_size_is_not_used(bench, tmp_path):
         "pass_kernel_code_sha256_16 = k\ndram_bytes_per_entry = 12.4230\n")
     assert bench.pass_traffic(2.0 ** 30) is None
 
-
-def test_the_committed_summary_is_of_the_present_kernel():
-    import bench
-    t = bench.pass_traffic(2.0 ** 32)
-    assert t is not None and 15.0 * 2.0 ** 32 < t < 17.0 * 2.0 ** 32
