@@ -431,11 +431,26 @@ private:
     int n_ = 0;
 };
 
+// Gates far from a unit scale: a singular value outside [1/2, 2]. Within it a step of
+// the sweep grows the boundary by 2^5 at most, 16 steps in a row by 2^80. Out of line:
+// inside plan_build it changes which products of the tables the compiler fuses on
+// aarch64, and with them the tables' last bits.
+__attribute__((noinline)) static bool far_from_unitary(const std::vector<M2>& gates) {
+    for (const M2& u : gates) {
+        double f = 0.0;  // sum and product of the squared singular values
+        for (const cd& z : u.a) f += std::norm(z);
+        const double det2 = std::norm(u.a[0] * u.a[3] - u.a[1] * u.a[2]);
+        const double root = std::sqrt(std::max(0.0, f * f - 4.0 * det2));
+        if (!(f + root <= 8.0 && f - root >= 0.5)) return true;
+    }
+    return false;
+}
+
 // Whether a zero entry stays zero whatever it is multiplied with: 0 x inf is not 0.
 // Every table that the device reads is finite in FP32 (gates of rows 0 and n-1 and of
 // the open band included), and no product of tables and no pass, which starts from
 // entries below 1, can leave FP32's range.
-static bool zeros_last(const Plan& P) {
+__attribute__((noinline)) static bool zeros_last(const Plan& P) {
     constexpr double LIMIT = 1e37;
     auto top = [](const void* v, size_t n) {  // largest magnitude of n floats; inf for inf and NaN
         const uint8_t* b = static_cast<const uint8_t*>(v);
@@ -682,16 +697,7 @@ int plan_build(Plan& P, int n, int d, const uint8_t* cliff, const uint8_t* tmask
         u = m2_mul(E, u);
     }
     auto U = [&](int q, int t) -> const M2& { return P.U[(size_t)t * n + q]; };
-    // Gates far from a unit scale: a singular value outside [1/2, 2]. Within it a
-    // step of the sweep grows the boundary by 2^5 at most, 16 steps in a row by 2^80.
-    P.wide_range = false;
-    for (const M2& u : P.U) {
-        double f = 0.0;  // sum and product of the squared singular values
-        for (const cd& z : u.a) f += std::norm(z);
-        const double det2 = std::norm(u.a[0] * u.a[3] - u.a[1] * u.a[2]);
-        const double root = std::sqrt(std::max(0.0, f * f - 4.0 * det2));
-        if (!(f + root <= 8.0 && f - root >= 0.5)) P.wide_range = true;
-    }
+    P.wide_range = far_from_unitary(P.U);
 
     // ---- entanglers: CZ, or diag(1, 1, 1, e^(i phi)) per gate (phi = pi is CZ exactly)
     P.W.assign((size_t)d * (n - 1), cd(-1.0, 0.0));
