@@ -629,14 +629,16 @@ __device__ void narrow_warp(const SmallParams& p, int b) {
 #pragma unroll
             for (int tg = 0; tg < H; ++tg) {
                 const int st = row * H + (fwd ? tg : H - 1 - tg);
-                const float4* g = reinterpret_cast<const float4*>(p.steps[st].g[tg == H - 1 ? xbit(row + 1) : 0]);
+                // 8-byte loads: a caller's workspace need not be aligned to 16
+                const float2* g = p.steps[st].g[tg == H - 1 ? xbit(row + 1) : 0];
                 const int ct = fwd ? tg - 1 : tg + 1;  // control bit (outside 0..H-1: none)
                 const bool cin = ct >= 0 && ct < H;
 #pragma unroll
                 for (int i = 0; i < NC; ++i) {
                     const int ap = tg < LB ? (int)(lane >> tg & 1u) : (i & 1);
                     const int c = !cin ? 0 : ct < LB ? (int)(lane >> (ct < 0 ? 0 : ct) & 1u) : (i >> 1);
-                    o[r][tg][i] = g[c * 2 + ap];
+                    const float2 g0 = g[c * 4 + ap * 2], g1 = g[c * 4 + ap * 2 + 1];
+                    o[r][tg][i] = make_float4(g0.x, g0.y, g1.x, g1.y);
                 }
             }
         }
