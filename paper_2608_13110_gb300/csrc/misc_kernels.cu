@@ -372,10 +372,12 @@ struct NarrowRun {
     static constexpr int ROW_CF = H * NARROW_CF;       // a row's packed coefficients
     static constexpr int CYCLE = 2 * H * 8;            // raw coefficients of two rows
     static constexpr int PRE = (CYCLE + T - 1) / T;    // of which a thread stages this many
-    // The last row's FP64 sum: as many strided partial sums as the few-bitstring form
-    // has threads, added in the same order in every form, so that an amplitude does
-    // not depend on how many bitstrings share the call.
-    static constexpr int GROUPS = narrow_threads(H, true) / T;
+    // The last row's FP64 sum has one grouping for both forms, so that an amplitude
+    // does not depend on how many bitstrings share the call: T0 sums (the threads of
+    // the many-bitstring form) of STRANDS strided sums each, a thread's own there and
+    // one per thread here when this form has more threads.
+    static constexpr int T0 = narrow_threads(H, false), STRANDS = narrow_threads(H, true) / T0, OWN = STRANDS * T0 / T;
+    static_assert(T == T0 || OWN == 1, "a thread holds all strands of its sum or one of them");
     float2* Bs;
     float2* cf;     // [2 buffers][2 rows][H][NARROW_CF]
     float* red;     // [2][NW]
@@ -556,10 +558,10 @@ struct NarrowRun {
             s = take_scale(turn);
         }
         const int xl = xb[p.n - 1] ? 1 : 0;
-        double ar[GROUPS] = {}, ai[GROUPS] = {};
-        for (int e0 = (int)t; e0 < N; e0 += GROUPS * T) {
+        double ar[OWN] = {}, ai[OWN] = {};
+        for (int e0 = (int)t; e0 < N; e0 += OWN * T) {
 #pragma unroll
-            for (int g = 0; g < GROUPS; ++g) {
+            for (int g = 0; g < OWN; ++g) {
                 const int e = e0 + g * T;
                 const float2 z = Bs[W::swz((uint32_t)e)];
                 const float2 v = cmul(make_float2(z.x * s, z.y * s), p.red_low[2 * e + xl]);
@@ -568,20 +570,29 @@ struct NarrowRun {
             }
         }
 #pragma unroll
-        for (int off = 16; off > 0; off >>= 1) {
+        for (int g = 1; g < OWN; ++g) { ar[0] += ar[g]; ai[0] += ai[g]; }
+        if constexpr (T > T0) {  // the other strands, through the coefficients' memory (no step is left)
+            double2* strand = reinterpret_cast<double2*>(cf);
+            if (t >= T0) strand[t - T0] = make_double2(ar[0], ai[0]);
+            sync();
+            if (t < T0)
 #pragma unroll
-            for (int g = 0; g < GROUPS; ++g) {
-                ar[g] += __shfl_xor_sync(0xffffffffu, ar[g], off);
-                ai[g] += __shfl_xor_sync(0xffffffffu, ai[g], off);
-            }
+                for (int g = 1; g < STRANDS; ++g) {
+                    const double2 o = strand[(g - 1) * T0 + t];
+                    ar[0] += o.x;
+                    ai[0] += o.y;
+                }
         }
 #pragma unroll
-        for (int g = 0; g < GROUPS; ++g)
-            if ((t & 31) == 0) redd[g * W::NW + (t >> 5)] = make_double2(ar[g], ai[g]);
+        for (int off = 16; off > 0; off >>= 1) {
+            ar[0] += __shfl_xor_sync(0xffffffffu, ar[0], off);
+            ai[0] += __shfl_xor_sync(0xffffffffu, ai[0], off);
+        }
+        if (t < T0 && (t & 31) == 0) redd[t >> 5] = make_double2(ar[0], ai[0]);
         sync();
         if (t == 0) {
             double2 tot = redd[0];
-            for (int i = 1; i < GROUPS * W::NW; ++i) { tot.x += redd[i].x; tot.y += redd[i].y; }
+            for (int i = 1; i < T0 / 32; ++i) { tot.x += redd[i].x; tot.y += redd[i].y; }
             const int Si = (int)max(-1000000LL, min(1000000LL, S));
             p.out[2 * b] = scalbn(tot.x, -Si);
             p.out[2 * b + 1] = scalbn(tot.y, -Si);
@@ -734,7 +745,7 @@ __device__ void narrow_warp(const SmallParams& p, int b) {
 }
 
 constexpr int narrow_smem(int h, bool few) {  // boundary, coefficients, reduction scratch of every warp
-    return h < 8 ? 0 : (8 << h) + 2 * 2 * h * NARROW_CF * 8 + (narrow_threads(h, true) / 32) * 16 +
+    return h < 8 ? 0 : (8 << h) + 2 * 2 * h * NARROW_CF * 8 + (narrow_threads(h, false) / 32) * 16 +
                            (narrow_threads(h, few) / 32) * 8;
 }
 
@@ -744,12 +755,13 @@ __device__ __forceinline__ void narrow_sweep(const SmallParams& p, int b, uint8_
         if (threadIdx.x < 32) narrow_warp<H>(p, b);
     } else {
         using R = NarrowRun<H, narrow_rw(H, FEW), WIDE>;
-        static_assert(R::T >= 32, "whole warps");
+        static_assert(R::T >= 32 && R::T0 >= 32, "whole warps");
+        static_assert((R::T - R::T0) * 16 <= 2 * 2 * R::ROW_CF * 8, "strands fit the coefficients' memory");
         if (threadIdx.x >= R::T) return;
         float2* Bs = reinterpret_cast<float2*>(smem);
         float2* cf = Bs + (1 << H);
-        double2* redd = reinterpret_cast<double2*>(cf + 2 * 2 * R::ROW_CF);  // [GROUPS][NW], then red [2][NW]
-        R r{Bs, cf, reinterpret_cast<float*>(redd + R::GROUPS * R::W::NW), p, p.bits + (int64_t)b * p.n, threadIdx.x, 0, {}};
+        double2* redd = reinterpret_cast<double2*>(cf + 2 * 2 * R::ROW_CF);  // [T0 / 32], then red [2][NW]
+        R r{Bs, cf, reinterpret_cast<float*>(redd + R::T0 / 32), p, p.bits + (int64_t)b * p.n, threadIdx.x, 0, {}};
         r.run(b, redd);
     }
 }
