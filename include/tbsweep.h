@@ -162,9 +162,10 @@ TB_API int tb_plan_create(int n, int d, const uint8_t* cliff, const uint8_t* tma
  * k >= 4 the join runs on the tensor cores and writes its product out of
  * place. When the boundary is wider than 2^33 entries, or the plan's
  * hbm_budget_bytes cannot hold two boundaries, the plan works in place: the
- * join runs in FP32 over the boundary itself and each late crossing writes
- * its output rows over its input rows (one boundary per prefix; 2^35
- * entries = 256 GiB at most). tb_workspace_bytes accounts for either.
+ * join runs in slices of rows through a scratch of one slice (in FP32 over
+ * the boundary itself for k < 4 or when the budget cannot hold the scratch)
+ * and each late crossing writes its output rows over its input rows (one
+ * boundary per prefix; 2^35 entries = 256 GiB at most). tb_workspace_bytes accounts for either.
  * tb_amplitudes_noalloc, batches and servers reject open plans (TB_EINVAL). */
 TB_API int tb_plan_create_open(int n, int d, const uint8_t* cliff, const uint8_t* tmask,
                                const tb_gate1q* extra, int n_extra, const tb_opts* opts, int k,

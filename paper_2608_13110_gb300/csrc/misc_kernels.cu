@@ -237,11 +237,12 @@ cudaError_t launch_finalize(const FinalizeParams& p, cudaStream_t st) {
 
 // Window bits at width h. few: the bitstrings fit one CTA per SM, so the length
 // of one sweep counts (fewer entries per thread, more warps); otherwise the
-// FP32 pipe counts (more steps per window). Measured with 1 / 256 / 512
-// bitstrings at n = 45 (us, before the last refinements): width 11 with RW = 2
-// 109 / 180 / 349, 3 124 / 151 / 308; width 12 with RW = 3 164 / 322 / 634,
-// 4 195 / 259 / 538; at widths 8 to 10 RW = 2 is the best for both (width 10:
-// 70 / 91 / 154, RW = 3 117 / 122 / 167).
+// FP32 pipe counts (more steps per window). Measured with 1 / 128 / 256 / 512 / 2048
+// bitstrings at n = 45 (us): width 10 with RW = 2 62 / 62 / 82 / 137 / 432, 3 86 / 105 /
+// 105 / 128 / 395; width 11 with RW = 2 100 / 101 / 161 / 312 / 1055, 3 88 / 111 / 136 /
+// 255 / 810; width 12 with RW = 3 142 / 144 / 250 / 485 / 1649, 4 142 / 180 / 239 / 488 /
+// 1782. At width 9 RW = 3 took 105 instead of 59 with one bitstring; at width 8 it
+// would leave half a warp.
 constexpr int narrow_rw(int h, bool few) { return h <= 10 ? 2 : h == 11 ? (few ? 2 : 3) : (few ? 3 : 4); }
 constexpr int narrow_threads(int h, bool few) { return h < 8 ? 32 : 1 << (h - narrow_rw(h, few) - 1); }
 
@@ -256,9 +257,9 @@ constexpr int narrow_threads(int h, bool few) { return h < 8 ? 32 : 1 << (h - na
 // to read and write shared memory behind a barrier. What bounds it: FP32 issue
 // (8 FMA per entry and step) once every SM has two warps per scheduler, the
 // chain of window moves and steps below that. n = 45, us for 1 / 256 / 2048
-// bitstrings, one step per barrier -> this form: width 8 147 / 154 / 458 ->
-// 49 / 49 / 109, width 10 240 / 279 / 1234 -> 62 / 82 / 434, width 11
-// 365 / 456 / 2353 -> 101 / 135 / 807, width 12 604 / 817 / 4771 -> 144 / 237 / 1770.
+// bitstrings, one step per barrier -> this form: width 8 144 / 154 / 457 ->
+// 49 / 49 / 109, width 10 236 / 279 / 1235 -> 62 / 82 / 432, width 11
+// 360 / 456 / 2355 -> 97 / 136 / 809, width 12 599 / 818 / 4775 -> 142 / 240 / 1782.
 // Power-of-two rescaling (exact) at every turn, folded into the next window's
 // first coefficients. Two things about that want gates near a unit scale: a
 // coefficient times the scale may leave FP32's range although its products do not

@@ -38,8 +38,9 @@
 // operands are all fresh registers takes 3 issue cycles instead of 2 (see
 // step_uniform) and two warps share a scheduler, which is why the loop reaches
 // 0.65 to 0.75 of the FMA rate. n=70, d=64 (width 32), 16 bitstrings: 0.36
-// amplitudes/s visiting every tile, 1.33 leaving the zeros out (27 % of the entries
-// visited; 0.75 of the HBM copy rate and 0.63 of the FMA rate on those).
+// amplitudes/s visiting every tile, 1.34 leaving the zeros out (27 % of the entries
+// visited: 0.76 of the HBM copy rate, and 0.59 of the FMA rate by the multiply-adds
+// that are executed).
 //
 // Rescaling: the producer of this pass's input left max(|re|,|im|) of its
 // output in maxs[slot]; this pass multiplies its input by 2^s (exact; folded

@@ -292,11 +292,12 @@ static void build_pass_steps(Plan& P) {
 // in nine per bit), and nothing later in the sweep undoes that before one of
 // the two bits is summed out. Support holds the affine space over GF(2) that
 // contains every nonzero entry: equations parity(address & mask) = value.
-// What it saves is the tiles no pass reads, computes or writes: with random
-// Clifford + T gates a pass visits 0.39-0.43 of its tiles at width 31, 0.44-0.52
-// at 28, 0.66-0.73 at 20, 0.9 at 16 (n = 70, d = 56, two bitstrings: 311 ms
-// visiting every tile, 134 ms; n = 30, d = 40, 32 bitstrings: 7.47 and 5.29 ms);
-// circuits without monomial gates visit every tile as before.
+// What it saves is the entries no pass reads, computes or writes: with random
+// Clifford + T gates a pass visits 0.35 of them at width 32, 0.42 at 28, 0.55 at 24,
+// 0.66 at 20 and 0.78 at 16 (means over 12 circuits; one circuit lies up to a
+// quarter off). Means over 8 circuits: n = 70, d = 56, two bitstrings 311 -> 134 ms;
+// n = 30, d = 40, 32 bitstrings 7.49 -> 4.10 ms with all of what stands here.
+// Circuits without monomial gates visit everything as before.
 class Support {
 public:
     static constexpr int TMP = 63;  // variable of the bit a step sums out
